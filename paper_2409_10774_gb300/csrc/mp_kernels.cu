@@ -1106,104 +1106,119 @@ __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 ? 2 : 1))
 // each ||<a>|| taken as the larger of its value now and the largest of the
 // converged increments so far (a cyclic load passes through zero means).
 // out[0] = err, out[1..4] = err_e, err_t, err_gamma, err_m, out[5] = status.
+// Run by warp 0 of the block, one lane per component, then one per field (the
+// chip's FP64 pipe is narrow and its latency long: with the fold below, an
+// iteration's reduction takes 18 us between events on a 64^3 cell where one
+// thread's took 26); out[0..5] are written by lanes 0..3.
+struct FinishScratch {
+  double mean[18], dev[18], stress[18], norm[4], ratio[4];
+};
 template <class R>
-__device__ void finish_err(const CellDev<R>& c, const double* s, int err_kind, double* out) {
-    const double iv = c.inv_nvox;
-    double me[9], mg[9], mt[9], mm[9];
-    for (int q = 0; q < 9; ++q) {
-      me[q] = s[8 + q] * iv;
-      mg[q] = s[17 + q] * iv;
-    }
-    // The transformed polarization was tau - tau_c = (t - T_c) - A0 (e - E) (T_c =
-    // c.tmean as read by pass A), so <t> = <tau - tau_c> + T_c + A0 (<e> - E) and
-    // likewise <m>; <t>, <m> then become the constants of the next iteration.
-    // In the increment form it was (t - t_prev) - A0 (e - e_prev), so the same
-    // formula holds with T_c = <t_prev> (the unrounded last mean) and
-    // <e_prev> = E.
-    const double lam = c.ref.lam, mu = c.ref.mu, kap = c.ref.kap;
-    const double al = c.ref.alpha, be = c.ref.beta, ga = c.ref.gamma;
-    double xe[9], xg[9];
-    for (int q = 0; q < 9; ++q) {
-      xe[q] = me[q] - (double)c.E[q];
-      xg[q] = mg[q] - (double)c.G[q];
-    }
-    const double tre = xe[0] + xe[4] + xe[8], trg = xg[0] + xg[4] + xg[8];
-    for (int k = 0; k < 3; ++k)
-      for (int l = 0; l < 3; ++l) {
-        const int i = 3 * k + l, j = 3 * l + k;
-        const double tc = c.delta_out ? c.tmean[i] : (double)(R)c.tmean[i];
-        const double mc = c.delta_out ? c.tmean[9 + i] : (double)(R)c.tmean[9 + i];
-        mt[i] = s[26 + i] * iv + tc + (mu + kap) * xe[i] + (mu - kap) * xe[j] + (k == l ? lam * tre : 0.0);
-        mm[i] = s[35 + i] * iv + mc + be * xg[i] + ga * xg[j] + (k == l ? al * trg : 0.0);
-      }
-    for (int q = 0; q < 9; ++q) {
-      c.tmean[q] = mt[q];
-      c.tmean[9 + q] = mm[q];
-    }
-    double ne = 0, ng = 0, nt = 0, nm = 0;
-    for (int q = 0; q < 9; ++q) {
-      ne += me[q] * me[q]; ng += mg[q] * mg[q]; nt += mt[q] * mt[q]; nm += mm[q] * mm[q];
-    }
-    ne = sqrt(ne); ng = sqrt(ng); nt = sqrt(nt); nm = sqrt(nm);
-    // magnitudes: the means now or, if larger, the largest of the converged
-    // increments so far (a cyclic load passing through a zero mean)
-    ne = fmax(ne, c.tmean[18]);
-    nt = fmax(nt, c.tmean[19]);
-    ng = fmax(ng, c.tmean[20]);
-    nm = fmax(nm, c.tmean[21]);
+__device__ __forceinline__ void finish_err(const CellDev<R>& c, const double* s, int err_kind, double* out,
+                                           FinishScratch& w) {
+  const int lane = threadIdx.x;
+  const double iv = c.inv_nvox;
+  const int lev = lane < 9 ? 0 : 1, i = lane - 9 * lev;  // lanes 0..17: component i of the macro / micro level
+  if (lane < 18) {
+    const double mean = s[8 + lane] * iv;
+    w.mean[lane] = mean;
+    w.dev[lane] = mean - (double)(lev == 0 ? c.E[i] : c.G[i]);
+  }
+  __syncwarp();
+  // The transformed polarization was tau - tau_c = (t - T_c) - A0 (e - E) (T_c =
+  // c.tmean as read by pass A), so <t> = <tau - tau_c> + T_c + A0 (<e> - E) and
+  // likewise <m>; <t>, <m> then become the constants of the next iteration.
+  // In the increment form it was (t - t_prev) - A0 (e - e_prev), so the same
+  // formula holds with T_c = <t_prev> (the unrounded last mean) and
+  // <e_prev> = E.
+  if (lane < 18) {
+    const int k = i / 3, l = i - 3 * k, j = 3 * l + k;
+    const double* x = w.dev + 9 * lev;
+    const double a = lev == 0 ? (double)c.ref.mu + (double)c.ref.kap : (double)c.ref.beta;
+    const double b = lev == 0 ? (double)c.ref.mu - (double)c.ref.kap : (double)c.ref.gamma;
+    const double d = lev == 0 ? (double)c.ref.lam : (double)c.ref.alpha;
+    const double tr = x[0] + x[4] + x[8];
+    const double tc = c.delta_out ? c.tmean[lane] : (double)(R)c.tmean[lane];
+    const double m = s[26 + lane] * iv + tc + a * x[i] + b * x[j] + (k == l ? d * tr : 0.0);
+    w.stress[lane] = m;
+    c.tmean[lane] = m;
+  }
+  __syncwarp();
+  // fields in the order e, t, gamma, m; magnitudes: the means now or, if
+  // larger, the largest of the converged increments so far (a cyclic load
+  // passing through a zero mean)
+  if (lane < 4) {
+    const double* v = ((lane & 1) ? w.stress : w.mean) + 9 * (lane >> 1);
+    double n = 0.0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) n += v[q] * v[q];
+    w.norm[lane] = fmax(sqrt(n), c.tmean[18 + lane]);
+  }
+  __syncwarp();
+  if (lane < 4) {
     const double h = c.h;
-    const double den[4] = {fmax(ne, h * ng), fmax(nt, nm / h), fmax(ng, ne / h), fmax(nm, h * nt)};
+    const double other = w.norm[lane ^ 2];  // the dimensional partner: e - gamma, t - m
+    const double den = fmax(w.norm[lane], (lane == 0 || lane == 3) ? h * other : other / h);
+    const double num = (err_kind == 0) ? s[lane] : s[4 + lane] * iv;
+    const double ea = den == 0.0 ? (num == 0.0 ? 0.0 : INFINITY) : num / den;
+    w.ratio[lane] = ea;
+    out[1 + lane] = ea;
+  }
+  __syncwarp();
+  if (lane == 0) {
     double err = 0.0;
-    for (int a = 0; a < 4; ++a) {
-      const double num = (err_kind == 0) ? s[a] : s[4 + a] * iv;
-      double ea;
-      if (den[a] == 0.0) ea = (num == 0.0) ? 0.0 : INFINITY;
-      else ea = num / den[a];
-      if (!(ea <= err)) err = ea;  // propagates NaN
-      out[1 + a] = ea;
-    }
+    for (int a = 0; a < 4; ++a)
+      if (!(w.ratio[a] <= err)) err = w.ratio[a];  // propagates NaN
     out[0] = err;
     out[5] = c.status ? (double)(*c.status) : 0.0;
+  }
 }
 
-// Fixed-order FP64 fold of `nparts` partial records (max for the first four
-// entries, sums for the rest; the block partials of a single cell, or a
-// batched cell's per-item records) by one block; the total lands in s[].
-// Thread (q, g) folds value q over the g-th of kFoldGroups contiguous record
-// ranges in record order (neighbouring q read neighbouring doubles), then
-// thread q folds the groups in order.
-constexpr int kFoldGroups = 5;  // 5 x 44 = 220 of the 256 threads
-__device__ __forceinline__ void fold_items(const double* partials, long long nparts, double* s,
-                                           double (*part)[kErrPartials]) {
+// Fixed-order FP64 fold of `nparts` records of NQ doubles (max for the first
+// NMAX values, sums for the rest) by one block of kFoldThreads; the total
+// lands in s[].  Thread (q, g) folds value q over the g-th contiguous range of
+// records in record order (neighbouring q read neighbouring doubles), then
+// thread q folds the ranges in order.  The loop is bound by the latency of its
+// loads and FP64 additions, so the ranges are as many as the block holds.
+constexpr int kFoldThreads = 1024;
+template <int NQ>
+constexpr int kFoldGroups = kFoldThreads / NQ;
+template <int NQ, int NMAX>
+__device__ __forceinline__ void fold_records(const double* __restrict__ records, long long nparts, double* s,
+                                             double (*part)[NQ]) {
+  constexpr int NG = kFoldGroups<NQ>;
   const int t = threadIdx.x;
-  if (t < kFoldGroups * kErrPartials) {
-    const int q = t % kErrPartials, g = t / kErrPartials;
-    const long long per = (nparts + kFoldGroups - 1) / kFoldGroups;
+  if (t < NG * NQ) {
+    const int q = t % NQ, g = t / NQ;
+    const long long per = (nparts + NG - 1) / NG;
     const long long b0 = (long long)g * per;
     const long long b1 = (b0 + per < nparts) ? b0 + per : nparts;
     double v = 0.0;
+#pragma unroll 8
     for (long long b = b0; b < b1; ++b) {
-      const double x = partials[b * kErrPartials + q];
-      v = (q < 4) ? fmax(v, x) : v + x;
+      const double x = records[b * NQ + q];
+      v = (q < NMAX) ? fmax(v, x) : v + x;
     }
     part[g][q] = v;
   }
   __syncthreads();
-  if (t < kErrPartials) {
+  if (t < NQ) {
     double v = part[0][t];
-    for (int g = 1; g < kFoldGroups; ++g) v = (t < 4) ? fmax(v, part[g][t]) : v + part[g][t];
+#pragma unroll
+    for (int g = 1; g < NG; ++g) v = (t < NMAX) ? fmax(v, part[g][t]) : v + part[g][t];
     s[t] = v;
   }
   __syncthreads();
 }
 
 template <class R>
-__global__ void __launch_bounds__(256) k_reduce_err(CellDev<R> c, const double* partials, int nparts,
-                                                    int err_kind, double* out) {
+__global__ void __launch_bounds__(kFoldThreads) k_reduce_err(CellDev<R> c, const double* partials, int nparts,
+                                                             int err_kind, double* out) {
   __shared__ double s[kErrPartials];
-  __shared__ double part[kFoldGroups][kErrPartials];
-  fold_items(partials, nparts, s, part);
-  if (threadIdx.x == 0) finish_err<R>(c, s, err_kind, out);
+  __shared__ double part[kFoldGroups<kErrPartials>][kErrPartials];
+  __shared__ FinishScratch fin;
+  fold_records<kErrPartials, 4>(partials, nparts, s, part);
+  if (threadIdx.x < 32) finish_err<R>(c, s, err_kind, out, fin);
 }
 
 // The same reduction, deciding the fixed-point loop on the device (Algorithm 2's
@@ -1214,15 +1229,16 @@ __global__ void __launch_bounds__(256) k_reduce_err(CellDev<R> c, const double* 
 // not tripped: out[7], out[8] hold the last low and its iteration, out[10]
 // the longest gap between lows, out[9] = 1 records a stop by the watch.
 template <class R>
-__global__ void __launch_bounds__(256) k_reduce_err_loop(CellDev<R> c, const double* partials, int nparts,
-                                                         int err_kind, double* out, double tol, int max_iter,
-                                                         double div_limit, int stag, int adapt,
-                                                         cudaGraphConditionalHandle handle) {
+__global__ void __launch_bounds__(kFoldThreads) k_reduce_err_loop(CellDev<R> c, const double* partials, int nparts,
+                                                                  int err_kind, double* out, double tol,
+                                                                  int max_iter, double div_limit, int stag,
+                                                                  int adapt, cudaGraphConditionalHandle handle) {
   __shared__ double s[kErrPartials];
-  __shared__ double part[kFoldGroups][kErrPartials];
-  fold_items(partials, nparts, s, part);
+  __shared__ double part[kFoldGroups<kErrPartials>][kErrPartials];
+  __shared__ FinishScratch fin;
+  fold_records<kErrPartials, 4>(partials, nparts, s, part);
+  if (threadIdx.x < 32) finish_err<R>(c, s, err_kind, out, fin);
   if (threadIdx.x == 0) {
-    finish_err<R>(c, s, err_kind, out);
     const int it = (int)out[6] + 1;
     out[6] = (double)it;
     const double err = out[0];
@@ -1242,7 +1258,6 @@ __global__ void __launch_bounds__(256) k_reduce_err_loop(CellDev<R> c, const dou
   }
 }
 
-// One block per entry: the cell's per-item partials in item order.
 // Algorithm 2's loop test for one batched cell after an iteration whose error
 // row is e (err, four terms, status), with the batched engine's FP32
 // stagnation watch; the same comparisons, in the same order and arithmetic,
@@ -1271,24 +1286,23 @@ __device__ void round_decide(RoundCtl& rc, const double* e) {
   rc.stop = stop ? 1 : 0;
 }
 
+// One block per entry: the cell's per-item partials.
 template <class R>
-__global__ void __launch_bounds__(256) k_reduce_err_multi(Work<R> w) {
+__global__ void __launch_bounds__(kFoldThreads) k_reduce_err_multi(Work<R> w) {
   __shared__ double s[kErrPartials];
-  __shared__ double part[kFoldGroups][kErrPartials];
+  __shared__ double part[kFoldGroups<kErrPartials>][kErrPartials];
+  __shared__ FinishScratch fin;
   __shared__ CellDev<R> cs;
   load_cell(cs, w.cells + w.act[blockIdx.x]);
   __syncthreads();
   RoundCtl* rc = cs.rctl;
   if (rc != nullptr && __ldcg(&rc->stop) != 0) return;  // uniform: one flag per block
-  fold_items(cs.ipart, cs.items_a, s, part);
-  if (threadIdx.x == 0) {
-    if (rc != nullptr) {
-      double* out = rc->rows + 8 * rc->rounds;
-      finish_err<R>(cs, s, cs.err_kind, out);
-      round_decide(*rc, out);
-    } else {
-      finish_err<R>(cs, s, cs.err_kind, cs.err_out);
-    }
+  fold_records<kErrPartials, 4>(cs.ipart, cs.items_a, s, part);
+  if (threadIdx.x < 32) {
+    double* out = rc != nullptr ? rc->rows + 8 * rc->rounds : cs.err_out;
+    finish_err<R>(cs, s, cs.err_kind, out, fin);
+    __syncwarp();
+    if (threadIdx.x == 0 && rc != nullptr) round_decide(*rc, out);
   }
 }
 
@@ -1478,45 +1492,43 @@ __global__ void __launch_bounds__(256) k_commit(CellDev<R> c0, Work<R> w, double
 }
 
 // The loading-history magnitudes of the error measure (cell scalars 18..21)
-// after a committed increment whose averages are row[0..35] (T, M, <e>, <gamma>).
+// after a committed increment whose averages are row[0..35] (T, M, <e>, <gamma>):
+// lanes 0..3 form ||<e>||, ||T||, ||<gamma>||, ||M||.
 __device__ __forceinline__ void update_history(const double* row, double* scalars) {
-  double n[4] = {0.0, 0.0, 0.0, 0.0};  // ||<e>||, ||T||, ||<gamma>||, ||M||
-  for (int q = 0; q < 9; ++q) {
-    n[0] += row[18 + q] * row[18 + q];
-    n[1] += row[q] * row[q];
-    n[2] += row[27 + q] * row[27 + q];
-    n[3] += row[9 + q] * row[9 + q];
+  const int a = threadIdx.x;
+  if (a < 4) {
+    const double* v = row + ((a & 1) ? 0 : 18) + 9 * (a >> 1);
+    double n = 0.0;
+    for (int q = 0; q < 9; ++q) n += v[q] * v[q];
+    scalars[18 + a] = fmax(scalars[18 + a], sqrt(n));
   }
-  for (int a = 0; a < 4; ++a) scalars[18 + a] = fmax(scalars[18 + a], sqrt(n[a]));
 }
 
-// Sum of the commit partials in a fixed order, divided by the voxel count.
-__global__ void k_reduce_avg(const double* partials, int nparts, double inv_nvox, double* out, double* scalars) {
+// Sum of commit records (block partials of a single cell, chunk records of a
+// batched one) in a fixed order, divided by the voxel count.  (The commit of a
+// 64^3 cell with its averages took 67.5 us with one thread per value, 52 so.)
+__device__ __forceinline__ void average_records(const double* records, long long n, double inv_nvox, double* out,
+                                                double* scalars) {
   __shared__ double row[kAvgPartials];
-  if (threadIdx.x < kAvgPartials) {
-    double s = 0.0;
-    for (int b = 0; b < nparts; ++b) s += partials[(long long)b * kAvgPartials + threadIdx.x];
-    out[threadIdx.x] = row[threadIdx.x] = s * inv_nvox;
-  }
+  __shared__ double part[kFoldGroups<kAvgPartials>][kAvgPartials];
+  fold_records<kAvgPartials, 0>(records, n, row, part);
+  if (threadIdx.x < kAvgPartials) out[threadIdx.x] = row[threadIdx.x] = row[threadIdx.x] * inv_nvox;
   __syncthreads();
-  if (threadIdx.x == 0) update_history(row, scalars);
+  update_history(row, scalars);
 }
 
-// One block per entry: the cell's chunk records in chunk order -> c.avg_out.
+__global__ void __launch_bounds__(kFoldThreads) k_reduce_avg(const double* partials, int nparts, double inv_nvox,
+                                                             double* out, double* scalars) {
+  average_records(partials, nparts, inv_nvox, out, scalars);
+}
+
+// One block per entry: the cell's chunk records -> c.avg_out.
 template <class R>
-__global__ void k_reduce_avg_multi(Work<R> w) {
+__global__ void __launch_bounds__(kFoldThreads) k_reduce_avg_multi(Work<R> w) {
   __shared__ CellDev<R> cs;
   load_cell(cs, w.cells + w.act[blockIdx.x]);
   __syncthreads();
-  __shared__ double row[kAvgPartials];
-  if (threadIdx.x < kAvgPartials) {
-    const long long n = (cs.nvox + 255) / 256;
-    double s = 0.0;
-    for (long long b = 0; b < n; ++b) s += cs.apart[b * kAvgPartials + threadIdx.x];
-    cs.avg_out[threadIdx.x] = row[threadIdx.x] = s * cs.inv_nvox;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) update_history(row, cs.tmean);
+  average_records(cs.apart, (cs.nvox + 255) / 256, cs.inv_nvox, cs.avg_out, cs.tmean);
 }
 
 // Final-state fields in FP64: e, gamma from `src` (prev or elast), t = h_t + A e,
@@ -1693,7 +1705,7 @@ cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* 
 template <class R>
 cudaError_t launch_reduce_err(const LaunchCfg& L, const CellDev<R>& c, const double* partials,
                               int err_kind, double* err_out, cudaStream_t st) {
-  k_reduce_err<R><<<1, 256, 0, st>>>(c, partials, L.grid_a, err_kind, err_out);
+  k_reduce_err<R><<<1, kFoldThreads, 0, st>>>(c, partials, L.grid_a, err_kind, err_out);
   return cudaGetLastError();
 }
 
@@ -1701,7 +1713,7 @@ template <class R>
 cudaError_t launch_reduce_err_loop(const LaunchCfg& L, const CellDev<R>& c, const double* partials, int err_kind,
                                    double* err_out, double tol, int max_iter, double div_limit, int stag,
                                    int adapt, cudaGraphConditionalHandle handle, cudaStream_t st) {
-  k_reduce_err_loop<R><<<1, 256, 0, st>>>(c, partials, L.grid_a, err_kind, err_out, tol, max_iter, div_limit,
+  k_reduce_err_loop<R><<<1, kFoldThreads, 0, st>>>(c, partials, L.grid_a, err_kind, err_out, tol, max_iter, div_limit,
                                           stag, adapt, handle);
   return cudaGetLastError();
 }
@@ -1731,7 +1743,7 @@ template <class R>
 cudaError_t launch_commit(const LaunchCfg& L, const CellDev<R>& c, double* partials, double* avg_out,
                           cudaStream_t st) {
   k_commit<R, false><<<L.grid_v, 256, kCommitSmem, st>>>(c, Work<R>{}, partials);
-  k_reduce_avg<<<1, 64, 0, st>>>(partials, L.grid_v, c.inv_nvox, avg_out, c.tmean);
+  k_reduce_avg<<<1, kFoldThreads, 0, st>>>(partials, L.grid_v, c.inv_nvox, avg_out, c.tmean);
   return cudaGetLastError();
 }
 
@@ -1749,7 +1761,7 @@ cudaError_t launch_multi_iteration(const MultiCfg<R>& m, cudaStream_t st) {
   if (m.items_a > 0)
     k_pass_a<R, kIter, true><<<m.grid_a, kThreads, m.smem_a, st>>>(CellDev<R>{}, m.wa, nullptr, nullptr,
                                                                     nullptr, nullptr, nullptr);
-  if (m.wa.n_act > 0) k_reduce_err_multi<R><<<m.wa.n_act, 256, 0, st>>>(m.wa);
+  if (m.wa.n_act > 0) k_reduce_err_multi<R><<<m.wa.n_act, kFoldThreads, 0, st>>>(m.wa);
   return cudaGetLastError();
 }
 
@@ -1767,7 +1779,7 @@ cudaError_t launch_multi_start(const MultiCfg<R>& m, cudaStream_t st) {
 template <class R>
 cudaError_t launch_multi_commit(const MultiCfg<R>& m, cudaStream_t st) {
   if (m.items_v > 0) k_commit<R, true><<<m.grid_v, 256, 0, st>>>(CellDev<R>{}, m.wv, nullptr);
-  if (m.wv.n_act > 0) k_reduce_avg_multi<R><<<m.wv.n_act, 64, 0, st>>>(m.wv);
+  if (m.wv.n_act > 0) k_reduce_avg_multi<R><<<m.wv.n_act, kFoldThreads, 0, st>>>(m.wv);
   return cudaGetLastError();
 }
 
