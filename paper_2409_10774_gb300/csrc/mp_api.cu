@@ -387,8 +387,7 @@ mp_status rve_setup(mp_rve* r, const mp_problem* p, cudaStream_t st) {
   MP_CK(ctx, cudaMemcpyAsync(r->phases.ptr, ph.data(), sizeof(PhaseDev<R>) * ph.size(),
                              cudaMemcpyHostToDevice, st));
   r->L = make_launch_cfg<R>(c, ctx->nsm);
-  c.rows_a = r->L.rows;
-  c.items_a = r->L.items_a;
+  use_launch_cfg(c, r->L);
   // per-block error partials for the largest pass-A grid any schedule can take
   // (pass A keeps at most two blocks on an SM)
   const size_t max_grid = std::max<size_t>((size_t)r->L.grid_a, 2 * (size_t)ctx->nsm);
@@ -459,8 +458,7 @@ mp_status twin_setup(mp_rve* r, cudaStream_t st) {
   MP_CK(ctx, cudaMemcpyAsync(r->phases64.ptr, ph.data(), sizeof(PhaseDev<double>) * ph.size(),
                              cudaMemcpyHostToDevice, st));
   r->L64 = make_launch_cfg<double>(c, ctx->nsm);
-  c.rows_a = r->L64.rows;
-  c.items_a = r->L64.items_a;
+  use_launch_cfg(c, r->L64);
   const size_t max_grid = std::max<size_t>((size_t)r->L64.grid_a, 2 * (size_t)ctx->nsm);
   if ((s = dalloc(ctx, r->partials64, sizeof(double) * kErrPartials * max_grid)) != MP_OK) return s;
   if ((s = dalloc(ctx, r->avgpart64, sizeof(double) * kAvgPartials * (size_t)r->L64.grid_v)) != MP_OK) return s;
@@ -580,8 +578,7 @@ mp_status rve_autotune(mp_rve* r, cudaStream_t st) {
   const std::array<int, 4> key{r->n[0], r->n[1], r->n[2], r->precision};
   auto apply = [&](int rows, int fused) {
     r->L = make_launch_cfg<R>(c, ctx->nsm, rows);
-    c.rows_a = r->L.rows;
-    c.items_a = r->L.items_a;
+    use_launch_cfg(c, r->L);
     r->use_fused = fused != 0;
   };
   {
@@ -1464,8 +1461,7 @@ mp_status green_apply_impl(mp_ctx* ctx, const int32_t n[3], double h, const doub
   if (st == MP_OK) {
     c.spec = reinterpret_cast<cpx<R>*>(spec.ptr);
     LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm);
-    c.rows_a = L.rows;
-    c.items_a = L.items_a;
+    use_launch_cfg(c, L);
     cudaError_t e = launch_green_apply<R>(L, c, (const R*)tau, (const R*)mu, (R*)e_out, (R*)g_out, cs,
                                           reinterpret_cast<int*>(ctl.ptr), ctx->nsm);
     int flag = 0;

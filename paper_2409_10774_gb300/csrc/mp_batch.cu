@@ -289,7 +289,7 @@ class Engine {
   // Arena bytes the request needs.
   size_t footprint(const Request& q) const {
     CellDev<R> c = shape_of(q);
-    LaunchCfg L = make_launch_cfg<R>(c, ctx_->nsm);
+    LaunchCfg L = make_launch_cfg<R>(c, ctx_->nsm, 0, true);
     return ArenaLayout<R>(q, L.items_a).total;
   }
 
@@ -531,7 +531,7 @@ class Engine {
   mp_status build_slot(Slot<R>& s, bool fresh) {
     Request* q = s.g.req;
     s.c = shape_of(*q);
-    s.L = make_launch_cfg<R>(s.c, ctx_->nsm);
+    s.L = make_launch_cfg<R>(s.c, ctx_->nsm, 0, true);
     const ArenaLayout<R> A(*q, s.L.items_a);
     s.bytes = A.total;
     s.arena = static_cast<unsigned char*>(pool_->take(A.total));
@@ -549,8 +549,7 @@ class Engine {
     c.tmean = reinterpret_cast<double*>(b + A.tmean);
     c.ipart = reinterpret_cast<double*>(b + A.ipart);
     c.apart = reinterpret_cast<double*>(b + A.apart);
-    c.rows_a = s.L.rows;
-    c.items_a = s.L.items_a;
+    use_launch_cfg(c, s.L);
     s.rows = reinterpret_cast<double*>(b + A.rows);
     s.fields = q->want_fields ? reinterpret_cast<double*>(b + A.fields) : nullptr;
     c.ref = ref_dev<R>(q->ref);
@@ -713,8 +712,8 @@ class Engine {
     fill(kFV0, l_init, [](const Slot<R>& s) { return (s.c.nvox + 255) / 256; });
     for (int i : l_iter) {
       const CellDev<R>& c = slots_[i].c;
-      m.smem_y = std::max(m.smem_y, c.n2 > 1 ? smem_line_pass<R>(c.n2) : (size_t)0);
-      m.smem_z = std::max(m.smem_z, smem_line_pass<R>(c.n3));
+      m.smem_y = std::max(m.smem_y, c.n2 > 1 ? smem_line<R>(c.n2, c.cols_y, 18) : (size_t)0);
+      m.smem_z = std::max(m.smem_z, smem_line<R>(c.n3, c.cols_z, c.n2 == 1 ? 18 : 12));
       m.smem_a = std::max(m.smem_a, smem_pass_a<R>(c.n1, c.rows_a));
     }
     for (int i : l_start) m.smem_a = std::max(m.smem_a, smem_pass_a<R>(slots_[i].c.n1, slots_[i].c.rows_a));

@@ -23,6 +23,23 @@ template <class R>
 __device__ __forceinline__ cpx<R> cadd(cpx<R> a, cpx<R> b) { return cmake<R>(a.x + b.x, a.y + b.y); }
 template <class R>
 __device__ __forceinline__ cpx<R> csub(cpx<R> a, cpx<R> b) { return cmake<R>(a.x - b.x, a.y - b.y); }
+// FP32 pairs: one packed instruction for both components (the same rounding).
+__device__ __forceinline__ cpx<float> cadd(cpx<float> a, cpx<float> b) {
+  cpx<float> c;
+  asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tadd.rn.f32x2 r, p, q;\n\t"
+      "mov.b64 {%0, %1}, r;\n\t}"
+      : "=f"(c.x), "=f"(c.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return c;
+}
+__device__ __forceinline__ cpx<float> csub(cpx<float> a, cpx<float> b) {
+  cpx<float> c;
+  asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tsub.rn.f32x2 r, p, q;\n\t"
+      "mov.b64 {%0, %1}, r;\n\t}"
+      : "=f"(c.x), "=f"(c.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return c;
+}
 template <class R>
 __device__ __forceinline__ cpx<R> cmul(cpx<R> a, cpx<R> b) {
   return cmake<R>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -102,6 +119,7 @@ template <class R>
 struct CellDev {
   int n1, n2, n3;
   int kx;                 // complex entries per spectral row: N1 / 2, or 1 when N1 == 1
+  unsigned kx_magic;      // ceil(2^32 / kx), 0 for kx == 1 (div_kx)
   long long nvox;         // N1 N2 N3
   long long nspec;        // kx N2 N3
   double h;
@@ -118,6 +136,7 @@ struct CellDev {
   AxisPlan<R> px, py, pz;
   R E[9], G[9];           // prescribed averages of the current step
   int* status;            // device status word: bit 0 = a bounded wait expired
+  int cols_y, cols_z;     // columns per tile of the y / z passes
   // batched (multi-cell) execution
   int rows_a;             // rows per pass-A work item
   long long items_a;      // pass-A work items
@@ -144,26 +163,15 @@ struct CellDev {
   RoundCtl* rctl;
 };
 
-// Columns per tile of the y / z passes for a transform length n: short
-// columns are grouped so that a tile holds about 256 points (the 288 threads
-// of a block then have a butterfly or a Green-operator point each); lengths
-// without a compile-time plan take one column per tile.
-__host__ __device__ constexpr int cols_per_tile(int n) {
-  return n == 16 ? 16 : n == 24 ? 10 : n == 32 ? 8 : n == 48 ? 5 : n == 64 ? 4 : n == 128 ? 2 : 1;
-}
 // Tiles of the y pass (columns (kz, kx), length N2) and of the z pass
 // (columns (ky, kx), length N3) of a cell.
 template <class R>
 __host__ __device__ inline long long tiles_y(const CellDev<R>& c) {
-  const long long cols = (long long)c.n3 * c.kx;
-  const int cpt = cols_per_tile(c.n2);
-  return (cols + cpt - 1) / cpt;
+  return ((long long)c.n3 * c.kx + c.cols_y - 1) / c.cols_y;
 }
 template <class R>
 __host__ __device__ inline long long tiles_z(const CellDev<R>& c) {
-  const long long cols = (long long)c.n2 * c.kx;
-  const int cpt = cols_per_tile(c.n3);
-  return (cols + cpt - 1) / cpt;
+  return ((long long)c.n2 * c.kx + c.cols_z - 1) / c.cols_z;
 }
 
 // The work of one multi-cell launch: entries e = 0..n_act-1 name cells

@@ -44,11 +44,17 @@ __device__ __forceinline__ void dft3(cpx<R>* v) {
 template <class R, int DIR>
 __device__ __forceinline__ void dft4(cpx<R>* v) {
   cpx<R> t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-  cpx<R> t2 = cadd(v[1], v[3]), t3 = rot90<R, DIR>(csub(v[1], v[3]));
+  cpx<R> t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
   v[0] = cadd(t0, t2);
   v[2] = csub(t0, t2);
-  v[1] = cadd(t1, t3);
-  v[3] = csub(t1, t3);
+  // t1 +- DIR i t3, component by component: no packing of the turned value
+  if constexpr (DIR < 0) {
+    v[1] = cmake<R>(t1.x + t3.y, t1.y - t3.x);
+    v[3] = cmake<R>(t1.x - t3.y, t1.y + t3.x);
+  } else {
+    v[1] = cmake<R>(t1.x - t3.y, t1.y + t3.x);
+    v[3] = cmake<R>(t1.x + t3.y, t1.y - t3.x);
+  }
 }
 
 template <class R, int DIR>
@@ -109,6 +115,137 @@ __device__ __forceinline__ void dft16(cpx<R>* v) {
     for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = t[k2];
   }
 }
+
+// 9-point DFT as 3 x 3: 3-point DFTs over x[3 n1 + n2], twiddles W_9^(n2 k1),
+// 3-point DFTs over n2; output index k1 + 3 k2.
+template <class R, int DIR>
+__device__ __forceinline__ void dft9(cpx<R>* v) {
+  cpx<R> a[3][3];
+#pragma unroll
+  for (int n2 = 0; n2 < 3; ++n2) {
+    cpx<R> t[3] = {v[n2], v[3 + n2], v[6 + n2]};
+    dft3<R, DIR>(t);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) a[n2][k1] = t[k1];
+  }
+  auto rot = [&](cpx<R> x, R cr, R si) {  // x * (cr + DIR i si)
+    return cmake<R>(x.x * cr - DIR * x.y * si, x.y * cr + DIR * x.x * si);
+  };
+  const R c1 = R(0.76604444311897803520239265055542), s1 = R(0.64278760968653932632264340990726);   // 2 pi / 9
+  const R c2 = R(0.17364817766693034885171662676931), s2 = R(0.98480775301220805936674302458952);   // 4 pi / 9
+  const R c4 = R(-0.93969262078590838405410927732473), s4 = R(0.34202014332566873304409961468226);  // 8 pi / 9
+  a[1][1] = rot(a[1][1], c1, s1);
+  a[1][2] = rot(a[1][2], c2, s2);
+  a[2][1] = rot(a[2][1], c2, s2);
+  a[2][2] = rot(a[2][2], c4, s4);
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    cpx<R> t[3] = {a[0][k1], a[1][k1], a[2][k1]};
+    dft3<R, DIR>(t);
+#pragma unroll
+    for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = t[k2];
+  }
+}
+
+template <class R, int DIR, int RADIX>
+__device__ __forceinline__ void dft(cpx<R>* v);
+
+// DFT of coprime factors A x B (the prime-factor map: no twiddles).  Input
+// n = (B n1 + A n2) mod A B, output k = (k1 B (B^-1 mod A) + k2 A (A^-1 mod B))
+// mod A B.
+template <class R, int DIR, int A, int B>
+__device__ __forceinline__ void dft_coprime(cpx<R>* v) {
+  constexpr auto inv = [](int x, int m) {
+    int r = 0;
+    while ((x * r) % m != 1 % m) ++r;
+    return r;
+  };
+  constexpr int N = A * B, CB = B * inv(B % A, A), CA = A * inv(A % B, B);
+  cpx<R> a[B][A];
+#pragma unroll
+  for (int n2 = 0; n2 < B; ++n2) {
+    cpx<R> t[A];
+#pragma unroll
+    for (int n1 = 0; n1 < A; ++n1) t[n1] = v[(B * n1 + A * n2) % N];
+    dft<R, DIR, A>(t);
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) a[n2][k1] = t[k1];
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < A; ++k1) {
+    cpx<R> t[B];
+#pragma unroll
+    for (int n2 = 0; n2 < B; ++n2) t[n2] = a[n2][k1];
+    dft<R, DIR, B>(t);
+#pragma unroll
+    for (int k2 = 0; k2 < B; ++k2) v[(k1 * CB + k2 * CA) % N] = t[k2];
+  }
+}
+
+template <class R, int DIR, int RADIX>
+__device__ __forceinline__ void dft(cpx<R>* v) {
+  if constexpr (RADIX == 1) return;
+  else if constexpr (RADIX == 2) dft2<R, DIR>(v);
+  else if constexpr (RADIX == 3) dft3<R, DIR>(v);
+  else if constexpr (RADIX == 4) dft4<R, DIR>(v);
+  else if constexpr (RADIX == 6) dft_coprime<R, DIR, 2, 3>(v);
+  else if constexpr (RADIX == 8) dft8<R, DIR>(v);
+  else if constexpr (RADIX == 9) dft9<R, DIR>(v);
+  else if constexpr (RADIX == 12) dft_coprime<R, DIR, 4, 3>(v);
+  else if constexpr (RADIX == 16) dft16<R, DIR>(v);
+  else {
+    static_assert(RADIX == 18, "no DFT of this radix");
+    dft_coprime<R, DIR, 2, 9>(v);
+  }
+}
+
+// Stages of a y / z line of length n: two for every length up to 324, so that
+// the line crosses shared memory once between them; lengths a thread holds
+// whole take one.
+struct LinePlan {
+  int count, r0, r1, r2;
+};
+__host__ __device__ constexpr LinePlan line_plan(int n) {
+  switch (n) {
+    case 1: case 2: case 4: case 6: case 8: case 12: case 16: case 18: return {1, n, 1, 1};
+    case 24: return {2, 6, 4, 1};
+    case 32: return {2, 8, 4, 1};
+    case 36: return {2, 6, 6, 1};
+    case 48: return {2, 8, 6, 1};
+    case 54: return {2, 9, 6, 1};
+    case 64: return {2, 8, 8, 1};
+    case 72: return {2, 9, 8, 1};
+    case 96: return {2, 12, 8, 1};
+    case 108: return {2, 12, 9, 1};
+    case 128: return {2, 16, 8, 1};
+    case 144: return {2, 12, 12, 1};
+    case 162: return {2, 18, 9, 1};
+    case 192: return {2, 16, 12, 1};
+    case 216: return {2, 18, 12, 1};
+    case 256: return {2, 16, 16, 1};
+    case 288: return {2, 18, 16, 1};
+    case 324: return {2, 18, 18, 1};
+    case 384: return {3, 8, 8, 6};
+    case 432: return {3, 9, 8, 6};
+    case 486: return {3, 9, 9, 6};
+    case 512: return {3, 8, 8, 8};
+    default: return {0, 1, 1, 1};
+  }
+}
+// Gap (complex values) after every r0 points of a two-stage column between its
+// stages: r0 lines and the gap advance the shared-memory banks as one line
+// does (a multiple of 16 complex values is a multiple of all banks, in FP32
+// and FP64), so a warp writes neighbouring butterflies like neighbouring points.
+__host__ __device__ constexpr int line_gap(int n, int lines) {
+  return line_plan(n).count == 2 ? (lines * 32 - lines * (line_plan(n).r0 - 1)) % 16 : 0;
+}
+// Complex values of such a column; an even number, so that tiles stay aligned.
+__host__ __device__ constexpr int line_pitch(int n, int lines) {
+  return (n * lines + n / line_plan(n).r0 * line_gap(n, lines) + 1) / 2 * 2;
+}
+// Complex entries of the table region of a line tile: n twiddles and n
+// frequencies, in whole 16-byte pieces.
+__host__ __device__ constexpr int line_table(int n) { return (n + (n + 1) / 2 + 1) / 2 * 2; }
 
 // Tiles are stored component-interleaved ("AoS"): element (row rr, point n,
 // component c) of a tile with `rows` rows of M points lives at
@@ -287,53 +424,6 @@ __device__ cpx<R>* tile_fft_x(cpx<R>* b0, cpx<R>* b1, int rows, const AxisPlan<R
     default:
       return tile_fft<R, DIR, 8>(b0, b1, rows, p, tw);
   }
-}
-
-// The y / z column transforms (twiddle stride 1) of a tile of
-// cols_per_tile(N) columns, 18 lines each, interleaved point by point: the
-// common lengths with the host's plan (radix 16 where it saves a stage, radix
-// 3 last) unrolled at compile time, others (one column per tile) through
-// tile_fft.
-template <class R, int DIR, int N>
-__device__ __forceinline__ cpx<R>* fft_yz_fixed(cpx<R>* b0, cpx<R>* b1, const cpx<R>* tw) {
-  constexpr int L = 18 * cols_per_tile(N);
-  auto sync_swap = [&]() {
-    __syncthreads();
-    cpx<R>* t = b0;
-    b0 = b1;
-    b1 = t;
-  };
-  if constexpr (N == 256) {
-    stage_fixed<R, DIR, 16, 1, 256, 1, L>(b0, b1, 1, tw); sync_swap();
-    stage_fixed<R, DIR, 16, 16, 256, 1, L>(b0, b1, 1, tw); sync_swap();
-  } else if constexpr (N == 128) {
-    stage_fixed<R, DIR, 16, 1, 128, 1, L>(b0, b1, 1, tw); sync_swap();
-    stage_fixed<R, DIR, 8, 16, 128, 1, L>(b0, b1, 1, tw); sync_swap();
-  } else if constexpr (N == 64) {
-    stage_fixed<R, DIR, 8, 1, 64, 1, L>(b0, b1, 1, tw); sync_swap();
-    stage_fixed<R, DIR, 8, 8, 64, 1, L>(b0, b1, 1, tw); sync_swap();
-  } else if constexpr (N == 48) {
-    stage_fixed<R, DIR, 16, 1, 48, 1, L>(b0, b1, 1, tw); sync_swap();
-    stage_fixed<R, DIR, 3, 16, 48, 1, L>(b0, b1, 1, tw); sync_swap();
-  } else if constexpr (N == 32) {
-    stage_fixed<R, DIR, 8, 1, 32, 1, L>(b0, b1, 1, tw); sync_swap();
-    stage_fixed<R, DIR, 4, 8, 32, 1, L>(b0, b1, 1, tw); sync_swap();
-  } else if constexpr (N == 24) {
-    stage_fixed<R, DIR, 8, 1, 24, 1, L>(b0, b1, 1, tw); sync_swap();
-    stage_fixed<R, DIR, 3, 8, 24, 1, L>(b0, b1, 1, tw); sync_swap();
-  } else {
-    static_assert(N == 16, "no compile-time plan for this length");
-    stage_fixed<R, DIR, 16, 1, 16, 1, L>(b0, b1, 1, tw); sync_swap();
-  }
-  return b0;
-}
-
-// NF > 0: the compile-time plan of length NF (cols_per_tile(NF) columns per
-// tile); otherwise the run-time plan p (one column per tile).
-template <class R, int DIR, int NF>
-__device__ cpx<R>* tile_fft_yz(cpx<R>* b0, cpx<R>* b1, const AxisPlan<R>& p, const cpx<R>* tw) {
-  if constexpr (NF > 0) return fft_yz_fixed<R, DIR, NF>(b0, b1, tw);
-  else return tile_fft<R, DIR, 16>(b0, b1, 1, p, tw);
 }
 
 }  // namespace mp

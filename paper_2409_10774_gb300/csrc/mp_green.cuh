@@ -110,4 +110,62 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
   }
 }
 
+// The same operator on the 12 reduced values of a point (mp_lines.cuh): in,
+// for l = 0..2, v[4l..4l+3] = A_l, T_l, B_l, M_l with f_l = A_l + i x3 T_l and
+// g_l = B_l + i x3 M_l; out u_l, i x3 u_l, phi_l, i x3 phi_l times `scale`.
+// v points to shared memory, 16-byte aligned; it moves in 16-byte pieces.
+template <class R>
+__device__ __forceinline__ void green_point_reduced(const RefDev<R>& A0, R x1, R x2, R x3, cpx<R>* v, R scale) {
+  struct __align__(16) Piece {
+    R w[16 / sizeof(R)];
+  };
+  const R xi[3] = {x1, x2, x3};
+  cpx<R> f[3], g[3];
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    __align__(16) cpx<R> q[4];
+#pragma unroll
+    for (int i = 0; i < (int)sizeof(q) / 16; ++i)
+      reinterpret_cast<Piece*>(q)[i] = reinterpret_cast<const Piece*>(v + 4 * l)[i];
+    f[l] = cmake<R>(fma(-x3, q[1].y, q[0].x), fma(x3, q[1].x, q[0].y));
+    g[l] = cmake<R>(fma(-x3, q[3].y, q[2].x), fma(x3, q[3].x, q[2].y));
+  }
+  const R k2 = x1 * x1 + x2 * x2 + x3 * x3;
+  const R ik2 = R(1) / k2;
+  const R a = (A0.mu + A0.kap) * k2;
+  const R b = A0.gamma * k2 + R(4) * A0.kap;
+  const R twok = R(2) * A0.kap;  // c = -i twok
+  const R iD = scale / (k2 * ((A0.mu + A0.kap) * A0.gamma * k2 + R(4) * A0.kap * A0.mu));
+  const R iL_u = scale * ik2 * ik2 / (A0.lam + R(2) * A0.mu);
+  const R iL_p = scale * ik2 / ((A0.alpha + A0.beta + A0.gamma) * k2 + R(4) * A0.kap);
+  cpx<R> xf = cmake<R>(R(0), R(0)), xg = cmake<R>(R(0), R(0));
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    xf = cadd(xf, cscale(f[l], xi[l]));
+    xg = cadd(xg, cscale(g[l], xi[l]));
+  }
+  cpx<R> cg[3], cf[3];  // xi x g, xi x f
+  cg[0] = csub(cscale(g[2], x2), cscale(g[1], x3));
+  cg[1] = csub(cscale(g[0], x3), cscale(g[2], x1));
+  cg[2] = csub(cscale(g[1], x1), cscale(g[0], x2));
+  cf[0] = csub(cscale(f[2], x2), cscale(f[1], x3));
+  cf[1] = csub(cscale(f[0], x3), cscale(f[2], x1));
+  cf[2] = csub(cscale(f[1], x1), cscale(f[0], x2));
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    const cpx<R> Pf = csub(f[l], cscale(xf, xi[l] * ik2));
+    const cpx<R> Pg = csub(g[l], cscale(xg, xi[l] * ik2));
+    const cpx<R> tu = cadd(cscale(Pf, b), cmuli(cscale(cg[l], twok)));
+    const cpx<R> tp = cadd(cscale(Pg, a), cmuli(cscale(cf[l], twok)));
+    __align__(16) cpx<R> q[4];
+    q[0] = cadd(cscale(xf, xi[l] * iL_u), cscale(tu, iD));
+    q[1] = cmuli(cscale(q[0], x3));
+    q[2] = cadd(cscale(xg, xi[l] * iL_p), cscale(tp, iD));
+    q[3] = cmuli(cscale(q[2], x3));
+#pragma unroll
+    for (int i = 0; i < (int)sizeof(q) / 16; ++i)
+      reinterpret_cast<Piece*>(v + 4 * l)[i] = reinterpret_cast<const Piece*>(q)[i];
+  }
+}
+
 }  // namespace mp

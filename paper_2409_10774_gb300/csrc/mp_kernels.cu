@@ -11,282 +11,25 @@
 // tau = t - A0 e, mu = m - B0 gamma, forward x transform.
 #include "mp_kernels.cuh"
 
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
+#include <set>
+#include <tuple>
+
 #include "mp_constitutive.cuh"
+#include "mp_device.cuh"
 #include "mp_fft.cuh"
 #include "mp_green.cuh"
 #include "mp_tma.cuh"
 
 namespace mp {
 
-// ------------------------------------------------------------------ helpers
-__device__ __forceinline__ float shfl_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ double shfl_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-template <class T>
-__device__ __forceinline__ T shfl_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-template <class R>
-__device__ __forceinline__ R signed_freq_scale(int k, int n, R two_pi_over_L) {
-  const int s = (k <= n / 2) ? k : k - n;
-  return two_pi_over_L * (R)s;
-}
-
 // 8 warps per block.  Registers are split between the SM's four sub-partitions
 // (16 K each), so with 2 blocks per SM (4 warps per sub-partition) a thread
 // may use up to 128 registers; a 9-warp block would cap it at 96.
 constexpr int kThreads = 256;
-// The y / z column passes: 18 components x 16 butterflies per round (a radix-16
-// stage of a 256-point line is exactly one round); their registers stay low.
-constexpr int kThreadsYZ = 288;
-// Shared memory per block on sm_103a (opt-in maximum) and the part of it the
-// dynamic tiles may use: the multi-cell kernels also hold a cell descriptor
-// and a few reduction words in static shared memory.
-constexpr size_t kSmemOptin = 227 * 1024;
-constexpr size_t kSmemStaticReserve = 2048;
-constexpr size_t kSmemBudget = kSmemOptin - kSmemStaticReserve;
-
-// Cooperative copy of a y / z tile of CPT columns (those below ncols; col0 is
-// the first), n points each, 18 complex values per (point, column): the values
-// of point p of tile column j sit at g + cofs[j] + p * stride (complex units)
-// and in the tile at ((p CPT + j) 18).  Loads are asynchronous 16-byte copies
-// (cp.async), so every thread keeps all of its loads in flight; the caller's
-// barrier follows cp_async_wait_all.
-template <class R, bool TO_SMEM, int CPT>
-__device__ __forceinline__ void copy_tile(cpx<R>* tile, cpx<R>* g, int n, long long col0, long long ncols,
-                                          long long stride, const long long* cofs) {
-  constexpr int W = 18 * (int)sizeof(cpx<R>) / 16;  // float4 per chunk
-  float4* t4 = reinterpret_cast<float4*>(tile);
-  const int total = n * CPT * W;
-  const int nj = (int)(ncols - col0 < CPT ? ncols - col0 : CPT);
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    const int row = i / W, w = i - row * W;
-    const int p = row / CPT, j = row - p * CPT;
-    if (j >= nj) continue;
-    float4* g4 = reinterpret_cast<float4*>(g + cofs[j] + p * stride) + w;
-    if (TO_SMEM) cp_async16(t4 + i, g4);
-    else *g4 = t4[i];
-  }
-  if (TO_SMEM) cp_async_wait_all();
-}
-
-// ------------------------------------------------------------------ multi-cell plumbing
-// Entry owning global item g: the last e with pre[e] <= g (binary search).
-__device__ __forceinline__ int find_entry(const long long* pre, int n, long long g) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= g) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// Cooperative copy of a cell descriptor into shared memory (callers fence with
-// barriers on both sides).
-template <class R>
-__device__ __forceinline__ void load_cell(CellDev<R>& dst, const CellDev<R>* src) {
-  static_assert(sizeof(CellDev<R>) % 4 == 0, "descriptor size");
-  const int* s4 = reinterpret_cast<const int*>(src);
-  int* d4 = reinterpret_cast<int*>(&dst);
-  for (int i = threadIdx.x; i < (int)(sizeof(CellDev<R>) / 4); i += blockDim.x) d4[i] = s4[i];
-}
-
-// Runs `body(cell, local_item)` over a launch's items: the single cell `c0`
-// (items 0..n0-1), or, for MULTI, every entry of `w` with its cell staged in
-// shared memory `cs` (reloaded when a block moves to the next cell).  A cell
-// whose round control says stop (a later round of a batched window after
-// its loop ended) has its items skipped; the flag only changes between
-// launches, so every thread of the block reads the same value.
-template <class R, bool MULTI, class Body>
-__device__ __forceinline__ void for_items(const CellDev<R>& c0, long long n0, const Work<R>& w,
-                                          CellDev<R>& cs, Body body) {
-  if constexpr (!MULTI) {
-    for (long long g = blockIdx.x; g < n0; g += gridDim.x) body(c0, g);
-  } else {
-    // contiguous ranges: a block's consecutive items mostly share a cell
-    const long long total = w.pre[w.n_act];
-    const long long per = (total + gridDim.x - 1) / gridDim.x;
-    const long long g0 = (long long)blockIdx.x * per;
-    const long long g1 = (g0 + per < total) ? g0 + per : total;
-    if (g0 >= g1) return;
-    int e = find_entry(w.pre, w.n_act, g0);
-    int cur = -1;
-    bool halted = false;
-    for (long long g = g0; g < g1; ++g) {
-      while (g >= w.pre[e + 1]) ++e;
-      const int slot = w.act[e];
-      if (slot != cur) {
-        __syncthreads();
-        load_cell(cs, w.cells + slot);
-        __syncthreads();
-        cur = slot;
-        halted = cs.rctl != nullptr && __ldcg(&cs.rctl->stop) != 0;
-      }
-      if (!halted) body(cs, g - w.pre[e]);
-    }
-  }
-}
-
-// ------------------------------------------------------------------ y pass
-// Shared memory of a y / z tile: two tiles of 18 cols_per_tile(n) lines of n
-// points, the axis' twiddle table (n entries) and the tile's column offsets.
-template <class R>
-size_t smem_line_pass(int n) {
-  return (2ull * 18 * cols_per_tile(n) + 1) * (size_t)n * sizeof(cpx<R>) + 16 * sizeof(long long);
-}
-
-// One tile = CPT consecutive columns (kz, kx), column index kz KX + kx, each
-// 18 lines of length N2.  NF > 0: N2 = NF with its compile-time plan and
-// CPT = cols_per_tile(NF); NF < 0: any length through the run-time plan, one
-// column per tile.
-template <class R, int DIR, int NF>
-__device__ __forceinline__ void fft_y_tile(const CellDev<R>& c, long long tile, unsigned char* smem) {
-  constexpr int CPT = NF > 0 ? cols_per_tile(NF) : 1;
-  cpx<R>* b0 = reinterpret_cast<cpx<R>*>(smem);
-  const int N = c.n2;
-  cpx<R>* b1 = b0 + 18 * CPT * N;
-  cpx<R>* tws = b1 + 18 * CPT * N;  // the axis' twiddle table, read from shared memory
-  long long* cofs = reinterpret_cast<long long*>(tws + N);
-  const int KX = c.kx;
-  const long long stride = (long long)KX * 18;
-  const long long ncols = (long long)c.n3 * KX, col0 = tile * CPT;
-  if (threadIdx.x < CPT) {
-    const long long col = col0 + threadIdx.x, kz = col / KX;
-    cofs[threadIdx.x] = (kz * N * KX + (col - kz * KX)) * 18;
-  }
-  for (int k = threadIdx.x; k < N; k += blockDim.x) tws[k] = c.py.tw[k];
-  __syncthreads();
-  copy_tile<R, true, CPT>(b0, c.spec, N, col0, ncols, stride, cofs);
-  __syncthreads();
-  cpx<R>* r = tile_fft_yz<R, DIR, NF>(b0, b1, c.py, tws);
-  copy_tile<R, false, CPT>(r, c.spec, N, col0, ncols, stride, cofs);
-  __syncthreads();
-}
-
-// Per-tile dispatch of the run-time-length kernels on the compile-time plans.
-template <class R, int DIR>
-__device__ __forceinline__ void fft_y_tile_any(const CellDev<R>& c, long long tile, unsigned char* smem) {
-  switch (c.n2) {
-    case 256: fft_y_tile<R, DIR, 256>(c, tile, smem); break;
-    case 128: fft_y_tile<R, DIR, 128>(c, tile, smem); break;
-    case 64: fft_y_tile<R, DIR, 64>(c, tile, smem); break;
-    case 48: fft_y_tile<R, DIR, 48>(c, tile, smem); break;
-    case 32: fft_y_tile<R, DIR, 32>(c, tile, smem); break;
-    case 24: fft_y_tile<R, DIR, 24>(c, tile, smem); break;
-    case 16: fft_y_tile<R, DIR, 16>(c, tile, smem); break;
-    default: fft_y_tile<R, DIR, -1>(c, tile, smem); break;
-  }
-}
-
-// NF > 0: compiled for one column length (its transform plan unrolled);
-// NF = 0: any length, dispatched per tile (multi-cell launches; every plan is
-// compiled into the one kernel, so it is given the registers of two blocks
-// per SM rather than spilling at three).
-template <class R, int DIR, bool MULTI, int NF>
-__global__ void __launch_bounds__(kThreadsYZ, NF > 0 ? 3 : 2) k_fft_y(CellDev<R> c0, Work<R> w) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ CellDev<R> cs;
-  for_items<R, MULTI>(c0, tiles_y(c0), w, cs, [&](const CellDev<R>& c, long long t) {
-    if constexpr (NF > 0) fft_y_tile<R, DIR, NF>(c, t, smem_raw);
-    else fft_y_tile_any<R, DIR>(c, t, smem_raw);
-  });
-}
-
-// ------------------------------------------------------------------ z pass + Green
-// One tile = CPT consecutive columns (ky, kx), column index ky KX + kx, each
-// 18 lines of length N3 (NF as for the y pass).
-template <class R, int NF>
-__device__ __forceinline__ void green_z_tile(const CellDev<R>& c, long long tile, unsigned char* smem) {
-  constexpr int CPT = NF > 0 ? cols_per_tile(NF) : 1;
-  cpx<R>* b0 = reinterpret_cast<cpx<R>*>(smem);
-  const int N = c.n3;
-  cpx<R>* b1 = b0 + 18 * CPT * N;
-  cpx<R>* tws = b1 + 18 * CPT * N;  // the axis' twiddle table, read from shared memory
-  long long* cofs = reinterpret_cast<long long*>(tws + N);
-  const int KX = c.kx;
-  const long long stride = (long long)c.n2 * KX * 18;
-  const long long ncols = (long long)c.n2 * KX, col0 = tile * CPT;
-  const R scale = (R)c.inv_nvox;
-  if (threadIdx.x < CPT) cofs[threadIdx.x] = (col0 + threadIdx.x) * 18;
-  for (int k = threadIdx.x; k < N; k += blockDim.x) tws[k] = c.pz.tw[k];
-  __syncthreads();
-  copy_tile<R, true, CPT>(b0, c.spec, N, col0, ncols, stride, cofs);
-  __syncthreads();
-  cpx<R>* r = tile_fft_yz<R, -1, NF>(b0, b1, c.pz, tws);
-  const bool even_y = (c.n2 % 2 == 0);
-  const int ky0 = (int)(col0 / KX), kx0 = (int)(col0 - (long long)ky0 * KX);
-  const int nj = (int)(ncols - col0 < CPT ? ncols - col0 : CPT);
-  for (int i = threadIdx.x; i < N * CPT; i += blockDim.x) {
-    const int kz = i / CPT, j = i - kz * CPT;
-    if (j >= nj) continue;
-    // column col0 + j = (ky, kx)
-    int kx = kx0 + j, ky = ky0;
-    if (CPT > 1) {
-      const int dy = kx / KX;
-      ky += dy;
-      kx -= dy * KX;
-    }
-    cpx<R>* pt = r + i * 18;  // the point's 18 values, updated in shared memory
-    // zero fluctuation on the Nyquist planes of y and z and at k = 0
-    const bool nyq = (even_y && ky == c.n2 / 2) || ((N % 2 == 0) && (kz == N / 2));
-    const bool zero = (kx == 0 && ky == 0 && kz == 0);
-    if (nyq || zero) {
-#pragma unroll
-      for (int q = 0; q < 18; ++q) pt[q] = cmake<R>(R(0), R(0));
-    } else {
-      const R x1 = c.n1 == 1 ? R(0) : c.two_pi_over_L[0] * (R)kx;
-      const R x2 = signed_freq_scale<R>(ky, c.n2, c.two_pi_over_L[1]);
-      const R x3 = signed_freq_scale<R>(kz, N, c.two_pi_over_L[2]);
-      green_point<R>(c.ref, x1, x2, x3, pt, scale);
-    }
-  }
-  __syncthreads();
-  cpx<R>* other = (r == b0) ? b1 : b0;
-  cpx<R>* o = tile_fft_yz<R, +1, NF>(r, other, c.pz, tws);
-  copy_tile<R, false, CPT>(o, c.spec, N, col0, ncols, stride, cofs);
-  __syncthreads();
-}
-
-template <class R>
-__device__ __forceinline__ void green_z_tile_any(const CellDev<R>& c, long long tile, unsigned char* smem) {
-  switch (c.n3) {
-    case 256: green_z_tile<R, 256>(c, tile, smem); break;
-    case 128: green_z_tile<R, 128>(c, tile, smem); break;
-    case 64: green_z_tile<R, 64>(c, tile, smem); break;
-    case 48: green_z_tile<R, 48>(c, tile, smem); break;
-    case 32: green_z_tile<R, 32>(c, tile, smem); break;
-    case 24: green_z_tile<R, 24>(c, tile, smem); break;
-    case 16: green_z_tile<R, 16>(c, tile, smem); break;
-    default: green_z_tile<R, -1>(c, tile, smem); break;
-  }
-}
-
-// The register file is split over the SM's four sub-partitions: 27 warps
-// (three 288-thread blocks) allow 72 registers per thread, which the FP32
-// single-length forms fit without spills; the others run two blocks per SM
-// (18 warps, 96 registers: a few spills cost less than one block per SM).
-template <class R, bool MULTI, int NF>
-__global__ void __launch_bounds__(kThreadsYZ, (sizeof(R) == 4 && NF > 0) ? 3 : 2)
-    k_green_z(CellDev<R> c0, Work<R> w) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ CellDev<R> cs;
-  for_items<R, MULTI>(c0, tiles_z(c0), w, cs, [&](const CellDev<R>& c, long long t) {
-    if constexpr (NF > 0) green_z_tile<R, NF>(c, t, smem_raw);
-    else green_z_tile_any<R>(c, t, smem_raw);
-  });
-}
-
 // ------------------------------------------------------------------ x pass (pass A)
 // Packed real transform of a row of N1 reals through a complex transform of
 // length M = N1 / 2: z[n] = x[2n] + i x[2n+1].
@@ -1030,16 +773,13 @@ __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 ? 2 : 1))
     }
     csm[4 * kThreads + threadIdx.x] = 0.0;
   }
-  for_items<R, MULTI>(c0, c0.items_a, w, cs, [&](const CellDev<R>& c, long long item) {
+  for_items<R, MULTI>(c0, c0.items_a, w, cs, [&](const CellDev<R>& c, long long item, bool fresh) {
     if (failed) {
       flag_timeout(c.status);  // every cell with a skipped item reports the failure
       return;
     }
-    // single cell: the block's first item stages the cell's tables; several
-    // cells: every item does (its cell may differ from the previous one's)
-    const bool reload = MULTI || item == (long long)blockIdx.x;
     if (!pass_a_item<R, MODE, MULTI>(c, item, smem_raw, parity, itm, tms, fin_tau, fin_mu, fout_e, fout_g,
-                                     reload)) {
+                                     fresh)) {
       failed = true;
       status = c.status;
       return;
@@ -1337,7 +1077,7 @@ template <class R, bool MULTI>
 __global__ void __launch_bounds__(256) k_init(CellDev<R> c0, Work<R> w) {
   __shared__ CellDev<R> cs;
   for_items<R, MULTI>(c0, (c0.nvox + 255) / 256, w, cs,
-                      [&](const CellDev<R>& c, long long chunk) { init_chunk<R>(c, chunk); });
+                      [&](const CellDev<R>& c, long long chunk, bool) { init_chunk<R>(c, chunk); });
 }
 
 // ------------------------------------------------------------------ commit
@@ -1464,7 +1204,7 @@ __global__ void __launch_bounds__(256) k_commit(CellDev<R> c0, Work<R> w, double
   if constexpr (!MULTI) {
     for (int i = threadIdx.x; i < kAvgPartials * (int)blockDim.x; i += blockDim.x) cols[i] = 0.0;
   }
-  for_items<R, MULTI>(c0, (c0.nvox + 255) / 256, w, cs, [&](const CellDev<R>& c, long long chunk) {
+  for_items<R, MULTI>(c0, (c0.nvox + 255) / 256, w, cs, [&](const CellDev<R>& c, long long chunk, bool) {
     commit_chunk<R, !MULTI>(c, chunk, chunk_sum, red, cols);
     if constexpr (MULTI) {
       if (threadIdx.x < kAvgPartials) c.apart[chunk * kAvgPartials + threadIdx.x] = chunk_sum[threadIdx.x];
@@ -1607,8 +1347,9 @@ size_t smem_pass_a(int n1, int rows) { return PassASmem<R>(n1, rows).total; }
 
 constexpr size_t kCommitSmem = (size_t)kAvgPartials * 256 * sizeof(double);  // single-cell commit columns
 
-// Raise each kernel's dynamic shared-memory limit to what its static shared
-// memory leaves of the opt-in maximum (at least kSmemBudget).
+// Raise the dynamic shared-memory limit of the kernels launched without a
+// resident_blocks call to what their static shared memory leaves of the
+// opt-in maximum (at least kSmemBudget).
 template <class R>
 static cudaError_t set_smem_attrs() {
   static bool done = false;
@@ -1628,18 +1369,6 @@ static cudaError_t set_smem_attrs() {
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kSmemOptin - fa.sharedSizeBytes));
   };
-  raise((const void*)k_fft_y<R, -1, false, 0>);
-  raise((const void*)k_fft_y<R, +1, false, 0>);
-  raise((const void*)k_fft_y<R, -1, false, 128>);
-  raise((const void*)k_fft_y<R, +1, false, 128>);
-  raise((const void*)k_fft_y<R, -1, false, 256>);
-  raise((const void*)k_fft_y<R, +1, false, 256>);
-  raise((const void*)k_fft_y<R, -1, true, 0>);
-  raise((const void*)k_fft_y<R, +1, true, 0>);
-  raise((const void*)k_green_z<R, false, 0>);
-  raise((const void*)k_green_z<R, false, 128>);
-  raise((const void*)k_green_z<R, false, 256>);
-  raise((const void*)k_green_z<R, true, 0>);
   raise((const void*)k_pass_a<R, kIter, false>);
   raise((const void*)k_pass_a<R, kStart, false>);
   raise((const void*)k_pass_a<R, kXFwd, false>);
@@ -1651,45 +1380,47 @@ static cudaError_t set_smem_attrs() {
   return e;
 }
 
+int resident_blocks(const void* fn, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int, size_t>, int> known;
+  static std::set<std::pair<int, const void*>> raised;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(dev, fn, threads, smem);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  if (!raised.count({dev, fn})) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kSmemOptin - fa.sharedSizeBytes)) != cudaSuccess)
+      return 1;
+    raised.insert({dev, fn});
+  }
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess) return 1;
+  if (per_sm < 1) per_sm = 1;
+  if (known.size() >= 4096) known.clear();
+  known[key] = per_sm;
+  return per_sm;
+}
+
 template <class R>
 int grid_for(const void* fn, int threads, size_t smem, long long work, int nsm) {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-  if (per_sm < 1) per_sm = 1;
-  long long g = (long long)per_sm * nsm;
-  if (work < g) g = work;
-  if (g < 1) g = 1;
-  return (int)g;
+  const long long g = std::min<long long>(work, (long long)resident_blocks(fn, threads, smem) * nsm);
+  return (int)std::max<long long>(g, 1);
 }
 
 template <class R>
 cudaError_t launch_fft_y(const LaunchCfg& L, const CellDev<R>& c, int dir, cudaStream_t st) {
-  cudaError_t e = set_smem_attrs<R>();
-  if (e != cudaSuccess) return e;
-  if (c.n2 > 1) {
-    const size_t sm = smem_line_pass<R>(c.n2);
-    if (dir < 0) {
-      if (c.n2 == 256) k_fft_y<R, -1, false, 256><<<L.grid_y, kThreadsYZ, sm, st>>>(c, Work<R>{});
-      else if (c.n2 == 128) k_fft_y<R, -1, false, 128><<<L.grid_y, kThreadsYZ, sm, st>>>(c, Work<R>{});
-      else k_fft_y<R, -1, false, 0><<<L.grid_y, kThreadsYZ, sm, st>>>(c, Work<R>{});
-    } else {
-      if (c.n2 == 256) k_fft_y<R, +1, false, 256><<<L.grid_y, kThreadsYZ, sm, st>>>(c, Work<R>{});
-      else if (c.n2 == 128) k_fft_y<R, +1, false, 128><<<L.grid_y, kThreadsYZ, sm, st>>>(c, Work<R>{});
-      else k_fft_y<R, +1, false, 0><<<L.grid_y, kThreadsYZ, sm, st>>>(c, Work<R>{});
-    }
-  }
-  return cudaGetLastError();
+  if (c.n2 == 1) return cudaSuccess;
+  return dir < 0 ? launch_line<R, kYForward>(c, L.grid_y, st) : launch_line<R, kYInverse>(c, L.grid_y, st);
 }
 
 template <class R>
 cudaError_t launch_green_z(const LaunchCfg& L, const CellDev<R>& c, cudaStream_t st) {
-  cudaError_t e = set_smem_attrs<R>();
-  if (e != cudaSuccess) return e;
-  const size_t sm = smem_line_pass<R>(c.n3);
-  if (c.n3 == 256) k_green_z<R, false, 256><<<L.grid_z, kThreadsYZ, sm, st>>>(c, Work<R>{});
-  else if (c.n3 == 128) k_green_z<R, false, 128><<<L.grid_z, kThreadsYZ, sm, st>>>(c, Work<R>{});
-  else k_green_z<R, false, 0><<<L.grid_z, kThreadsYZ, sm, st>>>(c, Work<R>{});
-  return cudaGetLastError();
+  return c.n2 == 1 ? launch_line<R, kZFull>(c, L.grid_z, st) : launch_line<R, kZReduced>(c, L.grid_z, st);
 }
 
 template <class R>
@@ -1752,12 +1483,9 @@ template <class R>
 cudaError_t launch_multi_iteration(const MultiCfg<R>& m, cudaStream_t st) {
   cudaError_t e = set_smem_attrs<R>();
   if (e != cudaSuccess) return e;
-  if (m.items_y > 0)
-    k_fft_y<R, -1, true, 0><<<m.grid_y, kThreadsYZ, m.smem_y, st>>>(CellDev<R>{}, m.wy);
-  if (m.items_z > 0)
-    k_green_z<R, true, 0><<<m.grid_z, kThreadsYZ, m.smem_z, st>>>(CellDev<R>{}, m.wz);
-  if (m.items_y > 0)
-    k_fft_y<R, +1, true, 0><<<m.grid_y, kThreadsYZ, m.smem_y, st>>>(CellDev<R>{}, m.wy);
+  if (m.items_y > 0 && (e = launch_line_multi<R, kYForward>(m.wy, m.grid_y, m.smem_y, st)) != cudaSuccess) return e;
+  if (m.items_z > 0 && (e = launch_line_multi<R, kZReduced>(m.wz, m.grid_z, m.smem_z, st)) != cudaSuccess) return e;
+  if (m.items_y > 0 && (e = launch_line_multi<R, kYInverse>(m.wy, m.grid_y, m.smem_y, st)) != cudaSuccess) return e;
   if (m.items_a > 0)
     k_pass_a<R, kIter, true><<<m.grid_a, kThreads, m.smem_a, st>>>(CellDev<R>{}, m.wa, nullptr, nullptr,
                                                                     nullptr, nullptr, nullptr);
@@ -1786,8 +1514,9 @@ cudaError_t launch_multi_commit(const MultiCfg<R>& m, cudaStream_t st) {
 template <class R>
 void multi_grids(MultiCfg<R>& m, int nsm) {
   set_smem_attrs<R>();
-  m.grid_y = grid_for<R>((const void*)k_fft_y<R, -1, true, 0>, kThreadsYZ, m.smem_y, m.items_y, nsm);
-  m.grid_z = grid_for<R>((const void*)k_green_z<R, true, 0>, kThreadsYZ, m.smem_z, m.items_z, nsm);
+  m.grid_y = std::min(line_multi_grid<R, kYForward>(m.items_y, m.smem_y, nsm),
+                      line_multi_grid<R, kYInverse>(m.items_y, m.smem_y, nsm));
+  m.grid_z = line_multi_grid<R, kZReduced>(m.items_z, m.smem_z, nsm);
   m.grid_a = grid_for<R>((const void*)k_pass_a<R, kIter, true>, kThreads, m.smem_a, m.items_a, nsm);
   m.grid_s = grid_for<R>((const void*)k_pass_a<R, kStart, true>, kThreads, m.smem_a, m.items_s, nsm);
   long long g = m.items_v < 8ll * nsm ? m.items_v : 8ll * nsm;
@@ -1820,9 +1549,9 @@ cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R*
     }
   }
   if (!fused) {
-    if (c.n2 > 1) k_fft_y<R, -1, false, 0><<<L.grid_y, kThreadsYZ, smem_line_pass<R>(c.n2), st>>>(c, Work<R>{});
-    k_green_z<R, false, 0><<<L.grid_z, kThreadsYZ, smem_line_pass<R>(c.n3), st>>>(c, Work<R>{});
-    if (c.n2 > 1) k_fft_y<R, +1, false, 0><<<L.grid_y, kThreadsYZ, smem_line_pass<R>(c.n2), st>>>(c, Work<R>{});
+    if ((e = launch_fft_y<R>(L, c, -1, st)) != cudaSuccess) return e;
+    if ((e = launch_green_z<R>(L, c, st)) != cudaSuccess) return e;
+    if ((e = launch_fft_y<R>(L, c, +1, st)) != cudaSuccess) return e;
   }
   k_pass_a<R, kXInv, false><<<L.grid_a, kThreads, sa, st>>>(c, Work<R>{}, nullptr, nullptr, nullptr, e_out, g_out);
   return cudaGetLastError();
@@ -1862,7 +1591,7 @@ template cudaError_t launch_convert<float, double>(const float*, double*, long l
 template cudaError_t launch_convert<double, float>(const double*, float*, long long, int, cudaStream_t);
 
 template <class R>
-LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted) {
+LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted, bool shared) {
   set_smem_attrs<R>();
   LaunchCfg L;
   // rows per pass-A item: about 256 voxels per block (or as asked), within the
@@ -1876,14 +1605,39 @@ LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted) {
   L.items_a = items;
   L.grid_a = grid_for<R>((const void*)k_pass_a<R, kIter, false>, kThreads, smem_pass_a<R>(c.n1, rows), items,
                          nsm);
-  const void* fy = c.n2 == 256   ? (const void*)k_fft_y<R, -1, false, 256>
-                   : c.n2 == 128 ? (const void*)k_fft_y<R, -1, false, 128>
-                                 : (const void*)k_fft_y<R, -1, false, 0>;
-  const void* fz = c.n3 == 256   ? (const void*)k_green_z<R, false, 256>
-                   : c.n3 == 128 ? (const void*)k_green_z<R, false, 128>
-                                 : (const void*)k_green_z<R, false, 0>;
-  L.grid_y = grid_for<R>(fy, kThreadsYZ, smem_line_pass<R>(c.n2), tiles_y(c), nsm);
-  L.grid_z = grid_for<R>(fz, kThreadsYZ, smem_line_pass<R>(c.n3), tiles_z(c), nsm);
+  // Columns per y / z tile: about 256 (FP32) or 128 (FP64) points for cells
+  // launched together.  A cell alone takes, in FP64, fewer where that would
+  // not give every SM two tiles (16^3: the three passes took 106 us in 8 tiles
+  // of 16 columns, 40 us in 128 of one; fewer columns than that only leave
+  // lanes of the FP64 pipe idle), and in FP32 the size that ends soonest: the
+  // tiles run in waves of what the SMs hold, and a wave costs its tile's
+  // points plus a fixed latency, about 100 points' worth (64^3: 11.9 us a pass
+  // in 512 tiles of four columns, which is one wave and an eighth, 10.6 us in
+  // 2048 of one).
+  auto columns = [&](int n, long long ncols) {
+    const int full = std::max(1, (sizeof(R) == 4 ? 256 : 128) / n);
+    if (shared) return full;
+    if (sizeof(R) == 8) return (int)std::min<long long>(full, std::max<long long>(1, ncols / (2 * nsm)));
+    int best = full;
+    double best_cost = INFINITY;
+    for (int cols = full; cols >= 1; --cols) {
+      const long long tiles = (ncols + cols - 1) / cols;
+      const long long slots = (long long)nsm * std::max(1, 800 / (cols * n));
+      const double cost = (double)((tiles + slots - 1) / slots) * (cols * n + 100.0);
+      if (cost < 0.97 * best_cost) {
+        best = cols;
+        best_cost = cost;
+      }
+    }
+    return best;
+  };
+  CellDev<R> t = c;
+  t.cols_y = L.cols_y = columns(c.n2, (long long)c.n3 * c.kx);
+  t.cols_z = L.cols_z = columns(c.n3, (long long)c.n2 * c.kx);
+  if (!shared) {
+    if (c.n2 > 1) L.grid_y = std::min(line_grid<R, kYForward>(t, nsm), line_grid<R, kYInverse>(t, nsm));
+    L.grid_z = c.n2 == 1 ? line_grid<R, kZFull>(t, nsm) : line_grid<R, kZReduced>(t, nsm);
+  }
   long long vb = (c.nvox + 255) / 256;
   L.grid_v = (int)(vb < 4ll * nsm ? vb : 4ll * nsm);
   return L;
@@ -1891,8 +1645,10 @@ LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted) {
 
 template <class R>
 bool sizes_fit(int n1, int n2, int n3) {
-  return smem_pass_a<R>(n1, 1) <= kSmemBudget && smem_line_pass<R>(n2) <= kSmemBudget &&
-         smem_line_pass<R>(n3) <= kSmemBudget;
+  // a y / z tile holds at least one whole column: two copies of its 18 lines
+  // and one more of a line's length for the tables
+  auto column = [](int n) { return 37 * (size_t)n * sizeof(cpx<R>) + 16 * sizeof(long long); };
+  return smem_pass_a<R>(n1, 1) <= kSmemBudget && column(n2) <= kSmemBudget && column(n3) <= kSmemBudget;
 }
 
 #define MP_INSTANTIATE(R)                                                                            \
@@ -1914,7 +1670,6 @@ bool sizes_fit(int n1, int n2, int n3) {
   template cudaError_t launch_multi_commit<R>(const MultiCfg<R>&, cudaStream_t);                      \
   template void multi_grids<R>(MultiCfg<R>&, int);                                                   \
   template size_t smem_pass_a<R>(int, int);                                                          \
-  template size_t smem_line_pass<R>(int);                                                            \
   template cudaError_t launch_fields<R>(const LaunchCfg&, const CellDev<R>&, int, double*, double*,   \
                                         double*, double*, double*, double*, cudaStream_t);           \
   template cudaError_t launch_green_apply<R>(const LaunchCfg&, const CellDev<R>&, const R*, const R*,  \
@@ -1923,7 +1678,7 @@ bool sizes_fit(int n1, int n2, int n3) {
                                                const R*, const R*, const R*, const R*, const R*,      \
                                                const R*, const double*, const double*, R*, R*,        \
                                                double*, double*, cudaStream_t);                       \
-  template LaunchCfg make_launch_cfg<R>(const CellDev<R>&, int, int);                                  \
+  template LaunchCfg make_launch_cfg<R>(const CellDev<R>&, int, int, bool);                                  \
   template bool sizes_fit<R>(int, int, int);
 
 MP_INSTANTIATE(float)

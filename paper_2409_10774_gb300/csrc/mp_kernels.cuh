@@ -2,6 +2,7 @@
 #pragma once
 
 #include "mp_common.cuh"
+#include "mp_fft.cuh"
 
 namespace mp {
 
@@ -9,17 +10,53 @@ struct LaunchCfg {
   int rows = 1;    // rows per pass-A work item
   long long items_a = 1;
   int grid_a = 1;  // pass-A grid (persistent, one error partial per block)
+  int cols_y = 1, cols_z = 1;  // columns per tile of the y / z passes
   int grid_y = 1;
   int grid_z = 1;
   int grid_v = 1;  // per-voxel kernels (init, commit, fields)
 };
 
 // rows_wanted > 0: that many rows per pass-A item (halved until the tile fits).
+// shared: the cell's work is launched together with other cells' (full y / z
+// tiles; a cell alone takes smaller ones rather than leave SMs idle).
 template <class R>
-LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted = 0);
+LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted = 0, bool shared = false);
+// Writes the configuration's item and tile sizes to the cell.
+template <class R>
+void use_launch_cfg(CellDev<R>& c, const LaunchCfg& L) {
+  c.rows_a = L.rows;
+  c.items_a = L.items_a;
+  c.cols_y = L.cols_y;
+  c.cols_z = L.cols_z;
+  c.kx_magic = c.kx > 1 ? (unsigned)(((1ull << 32) + c.kx - 1) / c.kx) : 0u;
+}
 // Whether the kernels' shared-memory tiles fit for this grid in precision R.
 template <class R>
 bool sizes_fit(int n1, int n2, int n3);
+
+// Blocks of `fn` an SM of the current device holds (at least 1), after letting
+// it use the shared memory its static part leaves of the opt-in maximum.
+// Answers are kept per kernel and shape: asking the runtime costs microseconds
+// and the component calls ask each time.
+int resident_blocks(const void* fn, int threads, size_t smem);
+
+// The line passes (mp_lines.cuh): y forward, y inverse, and z with the Green
+// operator on the reduced 12 fields or, for cells without a y pass, on all 18.
+enum LinePass { kYForward = 0, kYInverse = 1, kZReduced = 2, kZFull = 3 };
+// Shared memory of a tile of `cols` columns of n points: tables and two tiles
+// of `lines` lines (12 in the reduced z pass, else 18).
+template <class R>
+size_t smem_line(int n, int cols, int lines) {
+  return ((size_t)line_table(n) + ((size_t)lines * n + line_pitch(n, lines)) * cols) * sizeof(cpx<R>);
+}
+template <class R, int PASS>
+int line_grid(const CellDev<R>& c, int nsm);
+template <class R, int PASS>
+cudaError_t launch_line(const CellDev<R>& c, int grid, cudaStream_t st);
+template <class R, int PASS>
+int line_multi_grid(long long items, size_t smem, int nsm);
+template <class R, int PASS>
+cudaError_t launch_line_multi(const Work<R>& w, int grid, size_t smem, cudaStream_t st);
 
 // The kernels of one fixed-point iteration, one launch each (y pass dir -1 forward, +1 inverse).
 template <class R>
@@ -77,8 +114,6 @@ template <class R>
 cudaError_t launch_multi_commit(const MultiCfg<R>& m, cudaStream_t st);
 template <class R>
 size_t smem_pass_a(int n1, int rows);
-template <class R>
-size_t smem_line_pass(int n);
 template <class R>
 cudaError_t launch_fields(const LaunchCfg& L, const CellDev<R>& c, int from_elast, double* fe,
                           double* fg, double* ft, double* fm, double* fp, double* fq, cudaStream_t st);

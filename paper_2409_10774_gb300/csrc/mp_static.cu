@@ -115,8 +115,7 @@ mp_status run(mp_ctx* ctx, const int32_t n[3], double h, const double ref[6], co
     e = cudaMemcpyAsync(tw[a], host_tw[a], sizeof(cpx<R>) * n[a], cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm > 0 ? ctx->nsm : 1);
-    c.rows_a = L.rows;
-    c.items_a = L.items_a;
+    use_launch_cfg(c, L);
     e = launch_green_apply<R>(L, c, (const R*)tau, (const R*)mu, (R*)e_out, (R*)g_out, st);
   }
   int flag = 0;
