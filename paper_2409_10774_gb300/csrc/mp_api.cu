@@ -1376,7 +1376,39 @@ mp_status mp_solve(mp_ctx* ctx, const mp_problem* p, mp_result* res, void* strea
   return run;
 }
 
+}  // extern "C"
+
 // ------------------------------------------------------------------ components
+namespace {
+// A small phase table rides in the launch itself; a large one is copied to a
+// device buffer for the call.
+template <class R>
+mp_status radial_return_impl(mp_ctx* ctx, int32_t precision, int64_t count, const uint16_t* phase, int32_t n_phases,
+                             const mp_phase* phases, const void* e, const void* g, const void* e_n, const void* g_n,
+                             const void* t_n, const void* m_n, const double* p_n, const double* q_n, void* t, void* m,
+                             double* p, double* q, cudaStream_t cs) {
+  std::vector<PhaseDev<R>> ph(n_phases);
+  for (int k = 0; k < n_phases; ++k) ph[k] = phase_dev<R>(phases[k], precision == 2);
+  DevBuf tab;
+  cudaError_t err = cudaSuccess;
+  if (n_phases > max_table_phases()) {
+    const mp_status st = dalloc(ctx, tab, sizeof(PhaseDev<R>) * n_phases);
+    if (st != MP_OK) return st;
+    err = cudaMemcpyAsync(tab.ptr, ph.data(), tab.bytes, cudaMemcpyHostToDevice, cs);
+  }
+  if (err == cudaSuccess)
+    err = launch_radial_return<R>(ctx->nsm, count, phase, n_phases, ph.data(), (const PhaseDev<R>*)tab.ptr,
+                                  (const R*)e, (const R*)g, (const R*)e_n, (const R*)g_n, (const R*)t_n,
+                                  (const R*)m_n, p_n, q_n, (R*)t, (R*)m, p, q, cs);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(cs);
+  dfree(ctx, tab);
+  if (err != cudaSuccess) return set_error(ctx, MP_E_CUDA, "radial return: %s", cudaGetErrorString(err));
+  return MP_OK;
+}
+}  // namespace
+
+extern "C" {
+
 mp_status mp_radial_return(mp_ctx* ctx, int32_t precision, int64_t count, const uint16_t* phase,
                            int32_t n_phases, const mp_phase* phases, const void* e, const void* g,
                            const void* e_n, const void* g_n, const void* t_n, const void* m_n,
@@ -1393,37 +1425,11 @@ mp_status mp_radial_return(mp_ctx* ctx, int32_t precision, int64_t count, const 
     if (s != MP_OK) return set_error(ctx, s, "%s", msg.c_str());
   }
   MP_DEVICE_SCOPE(ctx);
-  mp_status st = MP_OK;
   cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-  DevBuf tab;
-  if (precision == 0) {
-    std::vector<PhaseDev<double>> ph(n_phases);
-    for (int k = 0; k < n_phases; ++k) ph[k] = phase_dev<double>(phases[k]);
-    if ((st = dalloc(ctx, tab, sizeof(PhaseDev<double>) * n_phases)) != MP_OK) return st;
-    cudaError_t e1 = cudaMemcpyAsync(tab.ptr, ph.data(), tab.bytes, cudaMemcpyHostToDevice, cs);
-    if (e1 == cudaSuccess)
-      e1 = launch_radial_return<double>(ctx->nsm, count, phase, (const PhaseDev<double>*)tab.ptr,
-                                        (const double*)e, (const double*)g, (const double*)e_n,
-                                        (const double*)g_n, (const double*)t_n, (const double*)m_n, p_n,
-                                        q_n, (double*)t, (double*)m, p, q, cs);
-    if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(cs);
-    dfree(ctx, tab);
-    if (e1 != cudaSuccess) return set_error(ctx, MP_E_CUDA, "radial return: %s", cudaGetErrorString(e1));
-  } else {
-    std::vector<PhaseDev<float>> ph(n_phases);
-    for (int k = 0; k < n_phases; ++k) ph[k] = phase_dev<float>(phases[k], precision == 2);
-    if ((st = dalloc(ctx, tab, sizeof(PhaseDev<float>) * n_phases)) != MP_OK) return st;
-    cudaError_t e1 = cudaMemcpyAsync(tab.ptr, ph.data(), tab.bytes, cudaMemcpyHostToDevice, cs);
-    if (e1 == cudaSuccess)
-      e1 = launch_radial_return<float>(ctx->nsm, count, phase, (const PhaseDev<float>*)tab.ptr,
-                                       (const float*)e, (const float*)g, (const float*)e_n,
-                                       (const float*)g_n, (const float*)t_n, (const float*)m_n, p_n,
-                                       q_n, (float*)t, (float*)m, p, q, cs);
-    if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(cs);
-    dfree(ctx, tab);
-    if (e1 != cudaSuccess) return set_error(ctx, MP_E_CUDA, "radial return: %s", cudaGetErrorString(e1));
-  }
-  return MP_OK;
+  return precision == 0 ? radial_return_impl<double>(ctx, precision, count, phase, n_phases, phases, e, g, e_n, g_n,
+                                                     t_n, m_n, p_n, q_n, t, m, p, q, cs)
+                        : radial_return_impl<float>(ctx, precision, count, phase, n_phases, phases, e, g, e_n, g_n,
+                                                    t_n, m_n, p_n, q_n, t, m, p, q, cs);
 }
 
 }  // extern "C"

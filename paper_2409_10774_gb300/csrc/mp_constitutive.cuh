@@ -18,19 +18,21 @@
 
 namespace mp {
 
-// 1 / sqrt(x) in FP64 for x > 0 by Newton's method on f(y) = 1/y^2 - x,
-// y <- y (3 - x y^2) / 2, from the single-precision hardware estimate
-// (relative error ~1e-7).  Two steps reach FP64 rounding.  Arguments outside
-// the single-precision normal range take the FP64 library path.
+// 1 / sqrt(x) in FP64 for x > 0 from the single-precision hardware estimate y
+// (relative error ~1e-7), with the residual e = 1 - x y^2: one Newton step
+// y (1 + e / 2) leaves a relative error near 1e-14; with the next term of
+// (1 - e)^(-1/2), y (1 + e / 2 + 3 e^2 / 8), it reaches FP64 rounding (five
+// FP64 operations; two Newton steps took seven, and the chip's FP64 pipe
+// bounds the material update).  Arguments outside the single-precision normal
+// range take the FP64 library path.
 // xf is x rounded to single precision (callers often have it at hand).
 template <int STEPS>
 __device__ __forceinline__ double rsqrt_newton(double x, float xf) {
   if (!(xf > 1e-36f && xf < 1e36f)) return 1.0 / sqrt(x);
-  double y = (double)rsqrtf(xf);
-  const double hx = 0.5 * x;
-#pragma unroll
-  for (int i = 0; i < STEPS; ++i) y = y * fma(-hx * y, y, 1.5);
-  return y;
+  const double y = (double)rsqrtf(xf);
+  const double e = fma(-x * y, y, 1.0);
+  if (STEPS == 1) return fma(0.5 * y, e, y);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // x >= 0 rounded toward zero to single precision (0 below the float normal
@@ -153,11 +155,12 @@ __device__ __forceinline__ void return_macro(const PhaseDev<R>& P, const R* e, c
   ft = R(1);
   const R vol = vol_of(t[0], t[4], t[8]);
   if (!P.elastic) {
-    // eq. equiv_stress on the trial deviator
+    // eq. equiv_stress on the trial deviator (its diagonal in one rounding,
+    // written out so that every kernel forms the same one)
     R s[9];
+    const R sum = (t[0] + t[4]) + t[8];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) s[i] = t[i];
-    s[0] -= vol; s[4] -= vol; s[8] -= vol;
+    for (int i = 0; i < 9; ++i) s[i] = i % 4 == 0 ? fma(R(-1.0 / 3.0), sum, t[i]) : t[i];
     const R teq2r = eq_sq(s, P.a1, P.a2, true);
     float f32;
     if (sizeof(R) == 4 && P.ret32) {

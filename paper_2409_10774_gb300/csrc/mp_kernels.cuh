@@ -122,12 +122,15 @@ cudaError_t launch_fields(const LaunchCfg& L, const CellDev<R>& c, int from_elas
 template <class R>
 cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R* tau, const R* mu,
                                R* e_out, R* g_out, cudaStream_t st, int* ctl = nullptr, int nsm = 0);
+// Algorithm 1 at `count` points.  The phase table is passed by value from
+// host_phases (n_phases <= max_table_phases()), or read from dev_phases.
 template <class R>
-cudaError_t launch_radial_return(int nsm, long long count, const uint16_t* phase,
-                                 const PhaseDev<R>* phases, const R* e, const R* g, const R* e_n,
-                                 const R* g_n, const R* t_n, const R* m_n, const double* p_n,
-                                 const double* q_n, R* t, R* m, double* p, double* q,
+cudaError_t launch_radial_return(int nsm, long long count, const uint16_t* phase, int n_phases,
+                                 const PhaseDev<R>* host_phases, const PhaseDev<R>* dev_phases, const R* e,
+                                 const R* g, const R* e_n, const R* g_n, const R* t_n, const R* m_n,
+                                 const double* p_n, const double* q_n, R* t, R* m, double* p, double* q,
                                  cudaStream_t st);
+int max_table_phases();
 
 // Fused spectral pass (y forward, z forward, Green operator, z inverse, y
 // inverse in one persistent launch; mp_spectral.cu) for FP32 cells whose y

@@ -94,6 +94,13 @@ __device__ __forceinline__ void fence_proxy_async() {
 __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
+// ... and of one 4- or 8-byte value (naturally aligned).
+template <class T>
+__device__ __forceinline__ void cp_async_value(T* dst_smem, const T* src) {
+  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "one value");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst_smem)), "l"(src), "n"((int)sizeof(T))
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 }  // namespace mp
