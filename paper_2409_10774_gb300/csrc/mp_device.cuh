@@ -7,12 +7,6 @@
 
 namespace mp {
 
-// Dynamic shared memory of a block: the opt-in maximum less a reserve for the
-// kernels' static shared memory.
-constexpr size_t kSmemOptin = 227 * 1024;
-constexpr size_t kSmemStaticReserve = 2048;
-constexpr size_t kSmemBudget = kSmemOptin - kSmemStaticReserve;
-
 // ------------------------------------------------------------------ helpers
 __device__ __forceinline__ float shfl_max(float v) {
 #pragma unroll

@@ -21,15 +21,34 @@
 #include "mp_constitutive.cuh"
 #include "mp_device.cuh"
 #include "mp_fft.cuh"
-#include "mp_green.cuh"
+#include "mp_lines.cuh"
 #include "mp_tma.cuh"
 
 namespace mp {
+
+// The line passes' own translation units compile them, except the z pass of
+// flat cells (N2 = 1), at the end of this one.
+#define MP_LINES_ELSEWHERE(R)                      \
+  MP_INSTANTIATE_LINE(R, kYForward, extern)        \
+  MP_INSTANTIATE_LINE(R, kYInverse, extern)        \
+  MP_INSTANTIATE_LINE(R, kZReduced, extern)        \
+  MP_INSTANTIATE_LINE_MULTI(R, kYForward, extern)  \
+  MP_INSTANTIATE_LINE_MULTI(R, kYInverse, extern)  \
+  MP_INSTANTIATE_LINE_MULTI(R, kZReduced, extern)
+MP_LINES_ELSEWHERE(float)
+MP_LINES_ELSEWHERE(double)
 
 // 8 warps per block.  Registers are split between the SM's four sub-partitions
 // (16 K each), so with 2 blocks per SM (4 warps per sub-partition) a thread
 // may use up to 128 registers; a 9-warp block would cap it at 96.
 constexpr int kThreads = 256;
+// Shared memory per block on sm_103a (opt-in maximum) and the part of it the
+// dynamic tiles may use: the multi-cell kernels also hold a cell descriptor
+// and a few reduction words in static shared memory.
+constexpr size_t kSmemOptin = 227 * 1024;
+constexpr size_t kSmemStaticReserve = 2048;
+constexpr size_t kSmemBudget = kSmemOptin - kSmemStaticReserve;
+
 // ------------------------------------------------------------------ x pass (pass A)
 // Packed real transform of a row of N1 reals through a complex transform of
 // length M = N1 / 2: z[n] = x[2n] + i x[2n+1].
@@ -1764,5 +1783,8 @@ bool sizes_fit(int n1, int n2, int n3) {
 
 MP_INSTANTIATE(float)
 MP_INSTANTIATE(double)
+
+MP_INSTANTIATE_LINE(float, kZFull)
+MP_INSTANTIATE_LINE(double, kZFull)
 
 }  // namespace mp

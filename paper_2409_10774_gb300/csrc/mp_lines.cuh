@@ -388,10 +388,15 @@ __device__ __forceinline__ void line_tile(const CellDev<R>& c, long long tile, c
 
 // One cell, one length.
 template <class R, int PASS, int N>
-__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS)) k_line(CellDev<R> c) {
+__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS)) k_fft_y(CellDev<R> c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const long long tiles = PASS < kZReduced ? tiles_y(c) : tiles_z(c);
-  for (long long t = blockIdx.x; t < tiles; t += gridDim.x)
+  for (long long t = blockIdx.x; t < tiles_y(c); t += gridDim.x)
+    line_tile<R, PASS, N>(c, t, reinterpret_cast<cpx<R>*>(smem_raw), t == (long long)blockIdx.x);
+}
+template <class R, int PASS, int N>
+__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS)) k_green_z(CellDev<R> c) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  for (long long t = blockIdx.x; t < tiles_z(c); t += gridDim.x)
     line_tile<R, PASS, N>(c, t, reinterpret_cast<cpx<R>*>(smem_raw), t == (long long)blockIdx.x);
 }
 
@@ -426,11 +431,16 @@ __global__ void __launch_bounds__(line_threads<R>(PASS), 2) k_line_multi(Work<R>
 }
 
 // ------------------------------------------------------------------ launches
+template <class R, int PASS, int N>
+const void* line_kernel() {
+  if constexpr (PASS < kZReduced) return (const void*)k_fft_y<R, PASS, N>;
+  else return (const void*)k_green_z<R, PASS, N>;
+}
 template <class R, int PASS>
 const void* line_kernel(int n) {
   switch (n) {
 #define MP_CASE(N) \
-  case N: return (const void*)k_line<R, PASS, N>;
+  case N: return line_kernel<R, PASS, N>();
     MP_LINE_LENGTHS(MP_CASE)
 #undef MP_CASE
     default: return nullptr;
@@ -477,10 +487,11 @@ cudaError_t launch_line_multi(const Work<R>& w, int grid, size_t smem, cudaStrea
   return cudaGetLastError();
 }
 
-#define MP_INSTANTIATE_LINES(R, PASS)                                               \
-  template int line_grid<R, PASS>(const CellDev<R>&, int);                          \
-  template cudaError_t launch_line<R, PASS>(const CellDev<R>&, int, cudaStream_t);  \
-  template int line_multi_grid<R, PASS>(long long, size_t, int);                    \
-  template cudaError_t launch_line_multi<R, PASS>(const Work<R>&, int, size_t, cudaStream_t);
+#define MP_INSTANTIATE_LINE(R, PASS, ...)                              \
+  __VA_ARGS__ template int line_grid<R, PASS>(const CellDev<R>&, int); \
+  __VA_ARGS__ template cudaError_t launch_line<R, PASS>(const CellDev<R>&, int, cudaStream_t);
+#define MP_INSTANTIATE_LINE_MULTI(R, PASS, ...)                              \
+  __VA_ARGS__ template int line_multi_grid<R, PASS>(long long, size_t, int); \
+  __VA_ARGS__ template cudaError_t launch_line_multi<R, PASS>(const Work<R>&, int, size_t, cudaStream_t);
 
 }  // namespace mp

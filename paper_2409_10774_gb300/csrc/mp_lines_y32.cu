@@ -1,9 +1,9 @@
-// The y passes in FP32.
+// The y passes of one cell in FP32.
 #include "mp_lines.cuh"
 
 namespace mp {
 
-MP_INSTANTIATE_LINES(float, kYForward)
-MP_INSTANTIATE_LINES(float, kYInverse)
+MP_INSTANTIATE_LINE(float, kYForward)
+MP_INSTANTIATE_LINE(float, kYInverse)
 
 }  // namespace mp

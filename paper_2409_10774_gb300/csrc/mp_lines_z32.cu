@@ -1,9 +1,8 @@
-// The z passes with the Green operator in FP32.
+// The z pass with the Green operator of one cell in FP32.
 #include "mp_lines.cuh"
 
 namespace mp {
 
-MP_INSTANTIATE_LINES(float, kZReduced)
-MP_INSTANTIATE_LINES(float, kZFull)
+MP_INSTANTIATE_LINE(float, kZReduced)
 
 }  // namespace mp

@@ -1,9 +1,8 @@
-// The z passes with the Green operator in FP64.
+// The z pass with the Green operator of one cell in FP64.
 #include "mp_lines.cuh"
 
 namespace mp {
 
-MP_INSTANTIATE_LINES(double, kZReduced)
-MP_INSTANTIATE_LINES(double, kZFull)
+MP_INSTANTIATE_LINE(double, kZReduced)
 
 }  // namespace mp
