@@ -1449,41 +1449,36 @@ mp_status green_apply_impl(mp_ctx* ctx, const int32_t n[3], double h, const doub
   c.inv_nvox = 1.0 / (double)c.nvox;
   for (int j = 0; j < 3; ++j) c.two_pi_over_L[j] = (R)(2.0 * M_PI / ((double)n[j] * h));
   c.ref = ref_dev<R>(ref);
-  DevBuf spec, tx, ty, tz, stat, ctl;
-  std::vector<cpx<R>> h1, h2, h3;
-  mp_status st = dalloc(ctx, spec, sizeof(cpx<R>) * 18 * (size_t)c.nspec);
-  if (st == MP_OK) st = dalloc(ctx, stat, sizeof(int) * 4);
-  if (st == MP_OK && cudaMemsetAsync(stat.ptr, 0, stat.bytes, cs) != cudaSuccess)
-    st = set_error(ctx, MP_E_CUDA, "cudaMemsetAsync failed");
-  c.status = reinterpret_cast<int*>(stat.ptr);
-  if (st == MP_OK) st = make_axis<R>(ctx, c.n1, true, c.px, tx, cs, h1);
-  if (st == MP_OK) st = make_axis<R>(ctx, c.n2, false, c.py, ty, cs, h2);
-  if (st == MP_OK) st = make_axis<R>(ctx, c.n3, false, c.pz, tz, cs, h3);
-  if constexpr (sizeof(R) == 4) {
-    if (st == MP_OK && spectral_fused_ok(c)) st = dalloc(ctx, ctl, sizeof(int) * spectral_ctl_ints(c.kx));
-    if (st == MP_OK && ctl.ptr && cudaMemsetAsync(ctl.ptr, 0, ctl.bytes, cs) != cudaSuccess)
-      st = set_error(ctx, MP_E_CUDA, "cudaMemsetAsync failed");
-  }
-  if (st == MP_OK) {
-    c.spec = reinterpret_cast<cpx<R>*>(spec.ptr);
-    LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm);
-    use_launch_cfg(c, L);
-    cudaError_t e = launch_green_apply<R>(L, c, (const R*)tau, (const R*)mu, (R*)e_out, (R*)g_out, cs,
-                                          reinterpret_cast<int*>(ctl.ptr), ctx->nsm);
-    int flag = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, stat.ptr, sizeof(int), cudaMemcpyDeviceToHost, cs);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
-    if (e != cudaSuccess) st = set_error(ctx, MP_E_CUDA, "green apply: %s", cudaGetErrorString(e));
-    else if (flag) st = set_error(ctx, MP_E_TIMEOUT, "green apply: a bounded device wait expired");
-  }
-  cudaStreamSynchronize(cs);
-  dfree(ctx, spec);
-  dfree(ctx, stat);
-  dfree(ctx, tx);
-  dfree(ctx, ty);
-  dfree(ctx, tz);
-  dfree(ctx, ctl);
-  return st;
+  // one device buffer (spectrum, then status, control words and twiddle
+  // tables) and one upload per call
+  bool fused = false;
+  if constexpr (sizeof(R) == 4) fused = spectral_fused_ok(c);
+  AxisPlan<R>* const plans[3] = {&c.px, &c.py, &c.pz};
+  static thread_local __align__(16) unsigned char image[kImageBytes];
+  size_t table[3];
+  const size_t image_bytes = operator_image<R>(n, plans, 4 + (fused ? spectral_ctl_ints(c.kx) : 0), image, table);
+  const size_t spec_bytes = (sizeof(cpx<R>) * 18 * (size_t)c.nspec + 255) / 256 * 256;
+  DevBuf buf;
+  mp_status st = dalloc(ctx, buf, spec_bytes + image_bytes);
+  if (st != MP_OK) return st;
+  unsigned char* meta = static_cast<unsigned char*>(buf.ptr) + spec_bytes;
+  c.spec = reinterpret_cast<cpx<R>*>(buf.ptr);
+  c.status = reinterpret_cast<int*>(meta);
+  for (int a = 0; a < 3; ++a) plans[a]->tw = reinterpret_cast<const cpx<R>*>(meta + table[a]);
+  LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm);
+  use_launch_cfg(c, L);
+  int flag = 0;
+  cudaError_t e = cudaMemcpyAsync(meta, image, image_bytes, cudaMemcpyHostToDevice, cs);
+  if (e == cudaSuccess)
+    e = launch_green_apply<R>(L, c, (const R*)tau, (const R*)mu, (R*)e_out, (R*)g_out, cs,
+                              fused ? c.status + 4 : nullptr, ctx->nsm);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c.status, sizeof(int), cudaMemcpyDeviceToHost, cs);
+  const cudaError_t es = cudaStreamSynchronize(cs);
+  if (e == cudaSuccess) e = es;
+  dfree(ctx, buf);
+  if (e != cudaSuccess) return set_error(ctx, MP_E_CUDA, "green apply: %s", cudaGetErrorString(e));
+  if (flag) return set_error(ctx, MP_E_TIMEOUT, "green apply: a bounded device wait expired");
+  return MP_OK;
 }
 }  // namespace
 

@@ -6,6 +6,8 @@
 #pragma once
 
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 #include <vector>
 
 #include "mp_common.cuh"
@@ -54,6 +56,26 @@ void axis_plan(int n, bool packed, AxisPlan<R>& p, cpx<R>* host_tw) {
   }
   p.tw = nullptr;
 }
+
+// What a Green-operator call uploads, as one image: `words` zeroed 32-bit words
+// (status and control), then the three axes' twiddle tables, 16-byte aligned.
+// Fills `image` (kImageBytes), the plans and the tables' byte offsets (the
+// plans' tw pointers are base + table[a]); returns the image's size.
+constexpr size_t kImageBytes = 32 * 1024;
+template <class R>
+size_t operator_image(const int32_t n[3], AxisPlan<R>* const plan[3], size_t words, unsigned char* image,
+                      size_t table[3]) {
+  size_t o = (words * 4 + 15) / 16 * 16;
+  std::memset(image, 0, o);
+  for (int a = 0; a < 3; ++a) {
+    table[a] = o;
+    axis_plan<R>(n[a], a == 0, *plan[a], reinterpret_cast<cpx<R>*>(image + o));
+    o += ((size_t)n[a] * sizeof(cpx<R>) + 15) / 16 * 16;
+  }
+  return o;
+}
+static_assert(4 * (4 + 2 + 2 * 256) + 16 + 3 * 512 * sizeof(cpx<double>) <= kImageBytes,
+              "the largest image: control words of 256 kx planes, three axes of 512 points");
 
 template <class R>
 void axis_tables(int n, bool packed, AxisPlan<R>& p, std::vector<cpx<R>>& host_tw) {

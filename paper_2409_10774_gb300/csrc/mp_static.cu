@@ -77,10 +77,6 @@ mp_status run(mp_ctx* ctx, const int32_t n[3], double h, const double ref[6], co
   mp_status s = scratch_for_device(ctx, &base);
   if (s != MP_OK) return s;
   unsigned char* b = static_cast<unsigned char*>(base);
-  int* status = reinterpret_cast<int*>(b);
-  cpx<R>* tw[3];
-  for (int a = 0; a < 3; ++a) tw[a] = reinterpret_cast<cpx<R>*>(b + 256 + (size_t)a * kMaxAxis * sizeof(cpx<double>));
-
   CellDev<R> c{};
   c.n1 = n[0];
   c.n2 = n[1];
@@ -102,24 +98,22 @@ mp_status run(mp_ctx* ctx, const int32_t n[3], double h, const double ref[6], co
   c.ref.beta = (R)ref[4];
   c.ref.gamma = (R)ref[5];
   c.spec = reinterpret_cast<cpx<R>*>(b + kTableRegion);
-  c.status = status;
-  AxisPlan<R>* plans[3] = {&c.px, &c.py, &c.pz};
-  // twiddle tables W_N^k = exp(-2 pi i k / N), built on the host stack and copied in
-  static thread_local cpx<R> host_tw[3][kMaxAxis];
-  for (int a = 0; a < 3; ++a) {
-    axis_plan<R>(n[a], a == 0, *plans[a], host_tw[a]);  // the plans every entry point uses
-    plans[a]->tw = tw[a];
-  }
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
-  for (int a = 0; a < 3 && e == cudaSuccess; ++a)
-    e = cudaMemcpyAsync(tw[a], host_tw[a], sizeof(cpx<R>) * n[a], cudaMemcpyHostToDevice, st);
+  c.status = reinterpret_cast<int*>(b);
+  // status word and twiddle tables W_N^k = exp(-2 pi i k / N), uploaded as one image
+  AxisPlan<R>* const plans[3] = {&c.px, &c.py, &c.pz};
+  static thread_local __align__(16) unsigned char image[kImageBytes];
+  static_assert(kImageBytes <= kTableRegion, "the image fits its region");
+  size_t table[3];
+  const size_t image_bytes = operator_image<R>(n, plans, 4, image, table);  // the plans every entry point uses
+  for (int a = 0; a < 3; ++a) plans[a]->tw = reinterpret_cast<const cpx<R>*>(b + table[a]);
+  cudaError_t e = cudaMemcpyAsync(b, image, image_bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm > 0 ? ctx->nsm : 1);
     use_launch_cfg(c, L);
     e = launch_green_apply<R>(L, c, (const R*)tau, (const R*)mu, (R*)e_out, (R*)g_out, st);
   }
   int flag = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, status, sizeof(int), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c.status, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(ctx, MP_E_CUDA, cudaGetErrorString(e));
   if (flag) return fail(ctx, MP_E_TIMEOUT, "mp_green_apply_static: a bounded device wait expired");
