@@ -389,8 +389,7 @@ mp_status rve_setup(mp_rve* r, const mp_problem* p, cudaStream_t st) {
   r->L = make_launch_cfg<R>(c, ctx->nsm);
   use_launch_cfg(c, r->L);
   // per-block error partials for the largest pass-A grid any schedule can take
-  // (pass A keeps at most two blocks on an SM)
-  const size_t max_grid = std::max<size_t>((size_t)r->L.grid_a, 2 * (size_t)ctx->nsm);
+  const size_t max_grid = (size_t)kPassABlocks * ctx->nsm;
   if ((s = dalloc(ctx, r->partials, sizeof(double) * kErrPartials * max_grid)) != MP_OK) return s;
   if ((s = dalloc(ctx, r->avgpart, sizeof(double) * kAvgPartials * (size_t)r->L.grid_v)) != MP_OK) return s;
   if ((s = dalloc(ctx, r->errout, sizeof(double) * 16)) != MP_OK) return s;
@@ -459,7 +458,7 @@ mp_status twin_setup(mp_rve* r, cudaStream_t st) {
                              cudaMemcpyHostToDevice, st));
   r->L64 = make_launch_cfg<double>(c, ctx->nsm);
   use_launch_cfg(c, r->L64);
-  const size_t max_grid = std::max<size_t>((size_t)r->L64.grid_a, 2 * (size_t)ctx->nsm);
+  const size_t max_grid = (size_t)kPassABlocks * ctx->nsm;
   if ((s = dalloc(ctx, r->partials64, sizeof(double) * kErrPartials * max_grid)) != MP_OK) return s;
   if ((s = dalloc(ctx, r->avgpart64, sizeof(double) * kAvgPartials * (size_t)r->L64.grid_v)) != MP_OK) return s;
   MP_CK(ctx, cudaStreamSynchronize(st));  // the host tables are locals

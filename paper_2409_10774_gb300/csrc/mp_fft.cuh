@@ -368,6 +368,28 @@ __device__ cpx<R>* tile_fft(cpx<R>* b0, cpx<R>* b1, int rows, const AxisPlan<R>&
   return in;
 }
 
+// Plan of a packed x transform of length m without compile-time stages of its
+// own: one stage (a thread holds the line) or two.  count 0: the run-time
+// radix plan.
+struct XPlan {
+  int count, r0, r1;
+};
+__host__ __device__ constexpr XPlan x_plan(int m) {
+  switch (m) {
+    case 2: case 3: case 4: case 6: case 9: return {1, m, 1};
+    case 18: return {2, 6, 3};
+    case 27: return {2, 9, 3};
+    case 36: return {2, 6, 6};
+    case 48: return {2, 8, 6};
+    case 54: return {2, 9, 6};
+    case 72: return {2, 9, 8};
+    case 81: return {2, 9, 9};
+    case 96: return {2, 12, 8};
+    case 108: return {2, 12, 9};
+    default: return {0, 1, 1};
+  }
+}
+
 // The x-axis transform inside pass A (twiddle stride 2: the table holds the
 // N1 = 2 M roots).  Common lengths are unrolled at compile time (radix <= 8,
 // radix 3 last, except 16 x 8 for M = 128 in FP32); others take tile_fft with

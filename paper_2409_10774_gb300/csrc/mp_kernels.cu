@@ -114,6 +114,168 @@ __device__ __forceinline__ void stage_first_inv_packed(const cpx<R>* __restrict_
   }
 }
 
+// ---- x transforms of the lengths in x_plan: the radices are compile-time, the
+// length is not (one body serves every length with that radix).  Rows hold M
+// points; butterfly j of a stage takes points j + r M / RADIX.
+template <class Body>
+__device__ __forceinline__ void x_butterflies(int rows, int nb, Body body) {
+  const unsigned magic = nb > 1 ? 0xffffffffu / (unsigned)nb + 1u : 0u;  // q / nb for q < 2^16
+  for (int idx = threadIdx.x; idx < rows * nb * 18; idx += blockDim.x) {
+    const int q = idx / 18, c = idx - q * 18;
+    const int rr = nb > 1 ? (int)__umulhi((unsigned)q, magic) : q;
+    body(c, rr, q - rr * nb);
+  }
+}
+
+// First inverse stage with the packed pre-step (as stage_first_inv_packed).
+template <class R, int RADIX>
+__device__ __forceinline__ void x_inv_first(const cpx<R>* X, cpx<R>* out, int rows, int M, const cpx<R>* tw) {
+  const int nb = M / RADIX;
+  x_butterflies(rows, nb, [=](int c, int rr, int j) {
+    const cpx<R>* x = X + rr * M * 18 + c;
+    cpx<R> v[RADIX];
+#pragma unroll
+    for (int r = 0; r < RADIX; ++r) {
+      const int k = j + r * nb;
+      cpx<R> a = x[k * 18], b = cconj(x[(k == 0 ? 0 : M - k) * 18]);
+      if (k == 0) {
+        a.y = R(0);
+        b = cmake<R>(R(0), R(0));
+      }
+      cpx<R> w = tw[k];
+      w.y = -w.y;  // W_N^-k
+      v[r] = cadd(cadd(a, b), cmuli(cmul(w, csub(a, b))));
+    }
+    dft<R, +1, RADIX>(v);
+    cpx<R>* dst = out + (rr * M + j * RADIX) * 18 + c;
+#pragma unroll
+    for (int r = 0; r < RADIX; ++r) dst[r * 18] = v[r];
+  });
+}
+// Last inverse stage (Ns = M / RADIX).
+template <class R, int RADIX>
+__device__ __forceinline__ void x_inv_last(const cpx<R>* in, cpx<R>* out, int rows, int M, const cpx<R>* tw) {
+  const int nb = M / RADIX;
+  x_butterflies(rows, nb, [=](int c, int rr, int j) {
+    const int o = (rr * M + j) * 18 + c;
+    cpx<R> v[RADIX];
+    v[0] = in[o];
+#pragma unroll
+    for (int r = 1; r < RADIX; ++r) v[r] = cmul(in[o + r * nb * 18], twiddle<R, +1>(tw, 2 * r * j));
+    dft<R, +1, RADIX>(v);
+#pragma unroll
+    for (int r = 0; r < RADIX; ++r) out[o + r * nb * 18] = v[r];
+  });
+}
+// First forward stage (Ns = 1).
+template <class R, int RADIX>
+__device__ __forceinline__ void x_fwd_first(const cpx<R>* in, cpx<R>* out, int rows, int M) {
+  const int nb = M / RADIX;
+  x_butterflies(rows, nb, [=](int c, int rr, int j) {
+    const cpx<R>* src = in + (rr * M + j) * 18 + c;
+    cpx<R> v[RADIX];
+#pragma unroll
+    for (int r = 0; r < RADIX; ++r) v[r] = src[r * nb * 18];
+    dft<R, -1, RADIX>(v);
+    cpx<R>* dst = out + (rr * M + j * RADIX) * 18 + c;
+#pragma unroll
+    for (int r = 0; r < RADIX; ++r) dst[r * 18] = v[r];
+  });
+}
+// Last forward stage with the packed post-step: butterflies u and Ns - u of a
+// line hold each other's partners (as x_forward_last_post; u = 0 and, for even
+// Ns, u = Ns / 2 are their own).  Ns = 1 is a whole transform.
+template <class R, int RADIX>
+__device__ __forceinline__ void x_fwd_last(const cpx<R>* in, cpx<R>* X, int rows, int M, const cpx<R>* tw) {
+  const int ns = M / RADIX, units = ns / 2 + 1;
+  x_butterflies(rows, units, [=](int c, int rr, int u) {
+    const cpx<R>* src = in + rr * M * 18 + c;
+    cpx<R>* dst = X + rr * M * 18 + c;
+    auto butterfly = [&](int j, cpx<R>(&v)[RADIX]) {
+      v[0] = src[j * 18];
+#pragma unroll
+      for (int r = 1; r < RADIX; ++r) {
+        v[r] = src[(j + r * ns) * 18];
+        if (ns > 1) v[r] = cmul(v[r], twiddle<R, -1>(tw, 2 * r * j));
+      }
+      dft<R, -1, RADIX>(v);
+    };
+    auto post = [&](int k, cpx<R> a, cpx<R> zp) {
+      const cpx<R> b = cconj(zp);
+      const cpx<R> sm = cadd(a, b), df = csub(a, b);
+      const cpx<R> wd = cmul(tw[k], df);
+      dst[k * 18] = cmake<R>(R(0.5) * (sm.x + wd.y), R(0.5) * (sm.y - wd.x));
+    };
+    cpx<R> v[RADIX];
+    butterfly(u, v);
+    if (u == 0) {
+#pragma unroll
+      for (int r = 0; r < RADIX; ++r) post(ns * r, v[r], v[(RADIX - r) % RADIX]);
+    } else if (2 * u == ns) {
+#pragma unroll
+      for (int r = 0; r < RADIX; ++r) post(u + ns * r, v[r], v[RADIX - 1 - r]);
+    } else {
+      cpx<R> w[RADIX];
+      butterfly(ns - u, w);
+#pragma unroll
+      for (int r = 0; r < RADIX; ++r) {
+        post(u + ns * r, v[r], w[RADIX - 1 - r]);
+        post(ns - u + ns * r, w[r], v[RADIX - 1 - r]);
+      }
+    }
+  });
+}
+
+// Inverse of packed rows in b0 by plan P (count > 0); returns the result's
+// buffer.  Ends with a barrier.
+template <class R>
+__device__ __forceinline__ cpx<R>* x_inv_planned(cpx<R>* b0, cpx<R>* b1, int rows, int M, const XPlan& P,
+                                                 const cpx<R>* tw) {
+  switch (P.r0) {
+    case 2: x_inv_first<R, 2>(b0, b1, rows, M, tw); break;
+    case 3: x_inv_first<R, 3>(b0, b1, rows, M, tw); break;
+    case 4: x_inv_first<R, 4>(b0, b1, rows, M, tw); break;
+    case 6: x_inv_first<R, 6>(b0, b1, rows, M, tw); break;
+    case 8: x_inv_first<R, 8>(b0, b1, rows, M, tw); break;
+    case 9: x_inv_first<R, 9>(b0, b1, rows, M, tw); break;
+    default: x_inv_first<R, 12>(b0, b1, rows, M, tw); break;
+  }
+  __syncthreads();
+  if (P.count == 1) return b1;
+  switch (P.r1) {
+    case 3: x_inv_last<R, 3>(b1, b0, rows, M, tw); break;
+    case 6: x_inv_last<R, 6>(b1, b0, rows, M, tw); break;
+    case 8: x_inv_last<R, 8>(b1, b0, rows, M, tw); break;
+    default: x_inv_last<R, 9>(b1, b0, rows, M, tw); break;
+  }
+  __syncthreads();
+  return b0;
+}
+// Forward of the packed rows in z, post-step included; the result replaces z.
+template <class R>
+__device__ __forceinline__ void x_fwd_planned(cpx<R>* z, cpx<R>* other, int rows, int M, const XPlan& P,
+                                              const cpx<R>* tw) {
+  const cpx<R>* in = z;  // one stage: each thread replaces the line it holds
+  if (P.count == 2) {
+    switch (P.r0) {
+      case 6: x_fwd_first<R, 6>(z, other, rows, M); break;
+      case 8: x_fwd_first<R, 8>(z, other, rows, M); break;
+      case 9: x_fwd_first<R, 9>(z, other, rows, M); break;
+      default: x_fwd_first<R, 12>(z, other, rows, M); break;
+    }
+    __syncthreads();
+    in = other;
+  }
+  switch (P.count == 2 ? P.r1 : P.r0) {
+    case 2: x_fwd_last<R, 2>(in, z, rows, M, tw); break;
+    case 3: x_fwd_last<R, 3>(in, z, rows, M, tw); break;
+    case 4: x_fwd_last<R, 4>(in, z, rows, M, tw); break;
+    case 6: x_fwd_last<R, 6>(in, z, rows, M, tw); break;
+    case 8: x_fwd_last<R, 8>(in, z, rows, M, tw); break;
+    default: x_fwd_last<R, 9>(in, z, rows, M, tw); break;
+  }
+}
+
 // Inverse x transform of packed rows: the spectral rows X in b0 -> the
 // packed real rows (returned: b0 or b1).  Ends with a barrier.
 template <class R>
@@ -165,6 +327,7 @@ __device__ cpx<R>* tile_fft_x_inv_packed(cpx<R>* b0, cpx<R>* b1, int rows, const
       stage_first_inv_packed<R, 8, 8>(b0, b1, rows, tw); sync_swap();
       return b0;
     default:
+      if (const XPlan P = x_plan(p.m); P.count > 0) return x_inv_planned<R>(b0, b1, rows, p.m, P, tw);
       x_inverse_pre<R>(b0, b1, rows, p.m, msh, tw);
       __syncthreads();
       return tile_fft<R, +1, 8>(b1, b0, rows, p, tw);
@@ -711,6 +874,10 @@ __device__ __forceinline__ bool pass_a_item(const CellDev<R>& c, long long item,
     if (M == 128) x_forward_last_post<R, 128, 8>(other, zbuf, nr, tws);
     else if (M == 64) x_forward_last_post<R, 64, 8>(other, zbuf, nr, tws);
     else x_forward_last_post<R, 32, 4>(other, zbuf, nr, tws);
+    X = zbuf;
+  } else if (const XPlan P = x_plan(M); packed && P.count > 0) {
+    // (the plan of a packed row; M = N1 / 2)
+    x_fwd_planned<R>(zbuf, (zbuf == b0) ? b1 : b0, nr, M, P, tws);
     X = zbuf;
   } else if (packed) {
     cpx<R>* other = (zbuf == b0) ? b1 : b0;
@@ -1543,7 +1710,7 @@ cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* 
                                cudaStream_t st) {
   cudaError_t e = set_smem_attrs<R>();
   if (e != cudaSuccess) return e;
-  k_pass_a<R, kIter, false><<<L.grid_a, kThreads, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
+  k_pass_a<R, kIter, false><<<L.grid_a, L.threads_a, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
       c, Work<R>{}, partials, nullptr, nullptr, nullptr, nullptr);
   return cudaGetLastError();
 }
@@ -1580,7 +1747,7 @@ cudaError_t launch_start(const LaunchCfg& L, const CellDev<R>& c, int first, cud
   cudaError_t e = set_smem_attrs<R>();
   if (e != cudaSuccess) return e;
   if (first) k_init<R, false><<<L.grid_v, 256, 0, st>>>(c, Work<R>{});
-  k_pass_a<R, kStart, false><<<L.grid_a, kThreads, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
+  k_pass_a<R, kStart, false><<<L.grid_a, L.threads_a, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
       c, Work<R>{}, nullptr, nullptr, nullptr, nullptr, nullptr);
   return cudaGetLastError();
 }
@@ -1655,7 +1822,7 @@ cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R*
   cudaError_t e = set_smem_attrs<R>();
   if (e != cudaSuccess) return e;
   const size_t sa = smem_pass_a<R>(c.n1, c.rows_a);
-  k_pass_a<R, kXFwd, false><<<L.grid_a, kThreads, sa, st>>>(c, Work<R>{}, nullptr, tau, mu, nullptr, nullptr);
+  k_pass_a<R, kXFwd, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, tau, mu, nullptr, nullptr);
   bool fused = false;
   if constexpr (sizeof(R) == 4) {
     if (ctl) {
@@ -1668,7 +1835,7 @@ cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R*
     if ((e = launch_green_z<R>(L, c, st)) != cudaSuccess) return e;
     if ((e = launch_fft_y<R>(L, c, +1, st)) != cudaSuccess) return e;
   }
-  k_pass_a<R, kXInv, false><<<L.grid_a, kThreads, sa, st>>>(c, Work<R>{}, nullptr, nullptr, nullptr, e_out, g_out);
+  k_pass_a<R, kXInv, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, nullptr, nullptr, e_out, g_out);
   return cudaGetLastError();
 }
 
@@ -1724,17 +1891,32 @@ template <class R>
 LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted, bool shared) {
   set_smem_attrs<R>();
   LaunchCfg L;
-  // rows per pass-A item: about 256 voxels per block (or as asked), within the
-  // shared-memory budget
-  int rows = rows_wanted > 0 ? rows_wanted : (c.n1 >= 256 ? 1 : 256 / c.n1);
-  while (rows > 1 && smem_pass_a<R>(c.n1, rows) > kSmemBudget) rows /= 2;
-  if ((long long)rows > (long long)c.n2 * c.n3) rows = (int)((long long)c.n2 * c.n3);
-  L.rows = rows;
+  // rows per pass-A item: about 256 voxels per block (FP64: 128, see below) or
+  // as asked, within the shared-memory budget; a cell alone takes fewer rows
+  // rather than leave SMs without an item, down to a warp of voxels
   const long long nrows = (long long)c.n2 * c.n3;
+  int rows = rows_wanted;
+  if (rows <= 0) {
+    const int want = sizeof(R) == 8 && !shared ? 128 : 256;
+    rows = c.n1 >= want ? 1 : want / c.n1;
+    if (!shared) {
+      const int least = (32 + c.n1 - 1) / c.n1;
+      rows = std::max(std::min(rows, least), (int)std::min<long long>(rows, (nrows + nsm - 1) / nsm));
+    }
+  }
+  while (rows > 1 && smem_pass_a<R>(c.n1, rows) > kSmemBudget) rows /= 2;
+  if ((long long)rows > nrows) rows = (int)nrows;
+  L.rows = rows;
   const long long items = (nrows + rows - 1) / rows;
   L.items_a = items;
-  L.grid_a = grid_for<R>((const void*)k_pass_a<R, kIter, false>, kThreads, smem_pass_a<R>(c.n1, rows), items,
-                         nsm);
+  // Threads: an item of up to 128 voxels keeps 128 busy.  In FP64 (up to 255
+  // registers a thread) that lets two blocks share an SM, so that one's
+  // material update fills the FP64 pipe while the other loads or waits at a
+  // barrier; an item too large for that keeps the SM's 256.
+  const size_t smem_a = smem_pass_a<R>(c.n1, rows);
+  L.threads_a = !shared && (long long)rows * c.n1 <= 128 && (sizeof(R) == 4 || 2 * smem_a <= kSmemOptin) ? 128 : kThreads;
+  L.grid_a = std::min(grid_for<R>((const void*)k_pass_a<R, kIter, false>, L.threads_a, smem_a, items, nsm),
+                      kPassABlocks * nsm);
   // Columns per y / z tile: about 256 (FP32) or 128 (FP64) points for cells
   // launched together.  A cell alone takes, in FP64, fewer where that would
   // not give every SM two tiles (16^3: the three passes took 106 us in 8 tiles

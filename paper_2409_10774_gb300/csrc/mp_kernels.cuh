@@ -9,6 +9,7 @@ namespace mp {
 struct LaunchCfg {
   int rows = 1;    // rows per pass-A work item
   long long items_a = 1;
+  int threads_a = 256;  // threads of a pass-A block
   int grid_a = 1;  // pass-A grid (persistent, one error partial per block)
   int cols_y = 1, cols_z = 1;  // columns per tile of the y / z passes
   int grid_y = 1;
@@ -16,6 +17,8 @@ struct LaunchCfg {
   int grid_v = 1;  // per-voxel kernels (init, commit, fields)
 };
 
+// Most pass-A blocks per SM of any launch configuration (one error partial each).
+constexpr int kPassABlocks = 4;
 // rows_wanted > 0: that many rows per pass-A item (halved until the tile fits).
 // shared: the cell's work is launched together with other cells' (full y / z
 // tiles; a cell alone takes smaller ones rather than leave SMs idle).

@@ -61,3 +61,13 @@ def test_green_apply_every_line_length(ctx, length, precision):
 @pytest.mark.parametrize("precision", [0, 1])
 def test_green_apply_flat_cells(ctx, n, precision):
     _check(ctx, n, precision)
+
+
+@pytest.mark.parametrize("length", LENGTHS)
+@pytest.mark.parametrize("precision", [0, 1])
+def test_green_apply_every_row_length(ctx, length, precision):
+    """The packed x transforms, several rows per item with the last item cut off."""
+    if precision == 0 and length > 324:
+        pytest.skip("an FP64 row longer than 324 voxels does not fit pass A's shared memory")
+    _check(ctx, (length, 6, 2), precision)
+    _check(ctx, (length, 1, 18), precision)
