@@ -389,8 +389,8 @@ mp_status rve_setup(mp_rve* r, const mp_problem* p, cudaStream_t st) {
   r->L = make_launch_cfg<R>(c, ctx->nsm);
   use_launch_cfg(c, r->L);
   // per-block error partials for the largest pass-A grid any schedule can take
-  const size_t max_grid = (size_t)kPassABlocks * ctx->nsm;
-  if ((s = dalloc(ctx, r->partials, sizeof(double) * kErrPartials * max_grid)) != MP_OK) return s;
+  if ((s = dalloc(ctx, r->partials, partials_bytes(ctx->nsm))) != MP_OK) return s;
+  MP_CK(ctx, cudaMemsetAsync(r->partials.ptr, 0, r->partials.bytes, st));
   if ((s = dalloc(ctx, r->avgpart, sizeof(double) * kAvgPartials * (size_t)r->L.grid_v)) != MP_OK) return s;
   if ((s = dalloc(ctx, r->errout, sizeof(double) * 16)) != MP_OK) return s;
   if ((s = dalloc(ctx, r->steprows, sizeof(double) * kAvgPartials * (size_t)r->n_steps)) != MP_OK) return s;
@@ -458,8 +458,8 @@ mp_status twin_setup(mp_rve* r, cudaStream_t st) {
                              cudaMemcpyHostToDevice, st));
   r->L64 = make_launch_cfg<double>(c, ctx->nsm);
   use_launch_cfg(c, r->L64);
-  const size_t max_grid = (size_t)kPassABlocks * ctx->nsm;
-  if ((s = dalloc(ctx, r->partials64, sizeof(double) * kErrPartials * max_grid)) != MP_OK) return s;
+  if ((s = dalloc(ctx, r->partials64, partials_bytes(ctx->nsm))) != MP_OK) return s;
+  MP_CK(ctx, cudaMemsetAsync(r->partials64.ptr, 0, r->partials64.bytes, st));
   if ((s = dalloc(ctx, r->avgpart64, sizeof(double) * kAvgPartials * (size_t)r->L64.grid_v)) != MP_OK) return s;
   MP_CK(ctx, cudaStreamSynchronize(st));  // the host tables are locals
   r->twin = true;
@@ -474,13 +474,25 @@ void set_load(CellDev<R>& c, const mp_rve* r, int s) {
   }
 }
 
-// The kernels of one fixed-point iteration (Algorithm 2's loop body), with
-// the loop-deciding error reduction when `handle` is given.
+// The error measure and loop bounds of the cell's next iterations.
+ErrTail err_tail(const mp_rve* r) {
+  ErrTail t{};
+  t.out = reinterpret_cast<double*>(r->errout.ptr);
+  t.err_kind = r->err_kind;
+  t.tol = r->tol;
+  t.div_limit = r->div_limit;
+  t.max_iter = r->loop_budget;
+  t.stag = r->loop_stag;
+  t.adapt = r->loop_adapt;
+  return t;
+}
+
+// The kernels of one fixed-point iteration (Algorithm 2's loop body), pass A
+// deciding the loop when `handle` is given.
 template <class R>
 cudaError_t launch_iteration_kernels(mp_rve* r, CellDev<R>& c, cudaStream_t st, const cudaGraphConditionalHandle* handle) {
   const LaunchCfg& L = cfg_of<R>(r);
   double* parts = partials_of<R>(r);
-  double* eout = reinterpret_cast<double*>(r->errout.ptr);
   cudaError_t e = cudaSuccess;
   bool fused = false;
   if constexpr (sizeof(R) == 4) fused = r->use_fused && r->ctl.ptr != nullptr;
@@ -491,12 +503,13 @@ cudaError_t launch_iteration_kernels(mp_rve* r, CellDev<R>& c, cudaStream_t st, 
     if (e == cudaSuccess) e = launch_green_z<R>(L, c, st);
     if (e == cudaSuccess) e = launch_fft_y<R>(L, c, +1, st);
   }
-  if (e == cudaSuccess) e = launch_pass_a_iter<R>(L, c, parts, st);
   if (e != cudaSuccess) return e;
-  if (handle)
-    return launch_reduce_err_loop<R>(L, c, parts, r->err_kind, eout, r->tol, r->loop_budget, r->div_limit,
-                                     r->loop_stag, r->loop_adapt, *handle, st);
-  return launch_reduce_err<R>(L, c, parts, r->err_kind, eout, st);
+  ErrTail tail = err_tail(r);
+  if (handle) {
+    tail.loop = 1;
+    tail.handle = *handle;
+  }
+  return launch_pass_a_iter<R>(L, c, parts, tail, st);
 }
 
 // Algorithm 2's while loop of one increment decided on the device: a graph
@@ -663,7 +676,6 @@ mp_status run_loop(mp_rve* r, CellDev<R>& c, int s, cudaStream_t st, int target,
       r->launches[MP_KC_GREEN_Z] += n;
     }
     r->launches[MP_KC_PASS_A] += n;
-    r->launches[MP_KC_REDUCE] += n;
   };
   auto classify = [&](const double* e) {
     if (e[5] != 0.0) o.status = MP_E_TIMEOUT;
@@ -699,7 +711,6 @@ mp_status run_loop(mp_rve* r, CellDev<R>& c, int s, cudaStream_t st, int target,
   int it_ref = 0;
   const LaunchCfg& L = cfg_of<R>(r);
   double* parts = partials_of<R>(r);
-  double* eout = reinterpret_cast<double*>(r->errout.ptr);
   const bool prof = r->profiling;
   auto mark = [&](int k, int end) {
     if (prof) cudaEventRecord(r->ev[2 * k + end], st);
@@ -727,17 +738,13 @@ mp_status run_loop(mp_rve* r, CellDev<R>& c, int s, cudaStream_t st, int target,
       mark(MP_KC_FFT_Y_INV, 1);
     }
     mark(MP_KC_PASS_A, 0);
-    MP_CK(ctx, launch_pass_a_iter<R>(L, c, parts, st));
+    MP_CK(ctx, launch_pass_a_iter<R>(L, c, parts, err_tail(r), st));
     mark(MP_KC_PASS_A, 1);
-    mark(MP_KC_REDUCE, 0);
-    MP_CK(ctx, launch_reduce_err<R>(L, c, parts, r->err_kind, eout, st));
-    mark(MP_KC_REDUCE, 1);
     MP_CK(ctx, cudaMemcpyAsync(r->err_host, r->errout.ptr, sizeof(double) * 6, cudaMemcpyDeviceToHost, st));
     MP_CK(ctx, cudaStreamSynchronize(st));
     count(1);
     if (prof) {
-      const int ks[6] = {MP_KC_FFT_Y_FWD, MP_KC_GREEN_Z, MP_KC_FFT_Y_INV, MP_KC_PASS_A, MP_KC_REDUCE,
-                         MP_KC_SPECTRAL};
+      const int ks[5] = {MP_KC_FFT_Y_FWD, MP_KC_GREEN_Z, MP_KC_FFT_Y_INV, MP_KC_PASS_A, MP_KC_SPECTRAL};
       for (int k : ks) {
         if (fused ? (k <= MP_KC_FFT_Y_INV) : (k == MP_KC_SPECTRAL)) continue;
         float ms = 0.f;

@@ -955,12 +955,204 @@ __device__ __forceinline__ bool pass_a_item(const CellDev<R>& c, long long item,
   return true;
 }
 
+// ------------------------------------------------------------------ iteration error
+// eq. err with eq. err_local (max) or eq. err_average (mean).  Denominators
+// ||<a>|| are floored by their dimensional partner through the voxel size h
+// (den_e >= h |<gamma>|, den_gamma >= |<e>| / h, den_t >= |<m>| / h,
+// den_m >= h |<t>|), since ||<gamma>|| = 0 whenever the mean curvature is zero,
+// each ||<a>|| taken as the larger of its value now and the largest of the
+// converged increments so far (a cyclic load passes through zero means).
+// out[0] = err, out[1..4] = err_e, err_t, err_gamma, err_m, out[5] = status.
+// Run by warp 0 of the block, one lane per component, then one per field (the
+// chip's FP64 pipe is narrow and its latency long: one thread took ~10 us);
+// out[0..5] are written by lanes 0..3.
+struct FinishScratch {
+  double mean[18], dev[18], stress[18], norm[4], ratio[4];
+};
+template <class R>
+__device__ __forceinline__ void finish_err(const CellDev<R>& c, const double* s, int err_kind, double* out,
+                                           FinishScratch& w) {
+  const int lane = threadIdx.x;
+  const double iv = c.inv_nvox;
+  const int lev = lane < 9 ? 0 : 1, i = lane - 9 * lev;  // lanes 0..17: component i of the macro / micro level
+  if (lane < 18) {
+    const double mean = s[8 + lane] * iv;
+    w.mean[lane] = mean;
+    w.dev[lane] = mean - (double)(lev == 0 ? c.E[i] : c.G[i]);
+  }
+  __syncwarp();
+  // The transformed polarization was tau - tau_c = (t - T_c) - A0 (e - E) (T_c =
+  // c.tmean as read by pass A), so <t> = <tau - tau_c> + T_c + A0 (<e> - E) and
+  // likewise <m>; <t>, <m> then become the constants of the next iteration.
+  // In the increment form it was (t - t_prev) - A0 (e - e_prev), so the same
+  // formula holds with T_c = <t_prev> (the unrounded last mean) and
+  // <e_prev> = E.
+  if (lane < 18) {
+    const int k = i / 3, l = i - 3 * k, j = 3 * l + k;
+    const double* x = w.dev + 9 * lev;
+    const double a = lev == 0 ? (double)c.ref.mu + (double)c.ref.kap : (double)c.ref.beta;
+    const double b = lev == 0 ? (double)c.ref.mu - (double)c.ref.kap : (double)c.ref.gamma;
+    const double d = lev == 0 ? (double)c.ref.lam : (double)c.ref.alpha;
+    const double tr = x[0] + x[4] + x[8];
+    const double tc = c.delta_out ? c.tmean[lane] : (double)(R)c.tmean[lane];
+    const double m = s[26 + lane] * iv + tc + a * x[i] + b * x[j] + (k == l ? d * tr : 0.0);
+    w.stress[lane] = m;
+    c.tmean[lane] = m;
+  }
+  __syncwarp();
+  // fields in the order e, t, gamma, m; magnitudes: the means now or, if
+  // larger, the largest of the converged increments so far (a cyclic load
+  // passing through a zero mean)
+  if (lane < 4) {
+    const double* v = ((lane & 1) ? w.stress : w.mean) + 9 * (lane >> 1);
+    double n = 0.0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) n += v[q] * v[q];
+    w.norm[lane] = fmax(sqrt(n), c.tmean[18 + lane]);
+  }
+  __syncwarp();
+  if (lane < 4) {
+    const double h = c.h;
+    const double other = w.norm[lane ^ 2];  // the dimensional partner: e - gamma, t - m
+    const double den = fmax(w.norm[lane], (lane == 0 || lane == 3) ? h * other : other / h);
+    const double num = (err_kind == 0) ? s[lane] : s[4 + lane] * iv;
+    const double ea = den == 0.0 ? (num == 0.0 ? 0.0 : INFINITY) : num / den;
+    w.ratio[lane] = ea;
+    out[1 + lane] = ea;
+  }
+  __syncwarp();
+  if (lane == 0) {
+    double err = 0.0;
+    for (int a = 0; a < 4; ++a)
+      if (!(w.ratio[a] <= err)) err = w.ratio[a];  // propagates NaN
+    out[0] = err;
+    out[5] = c.status ? (double)__ldcg(c.status) : 0.0;
+  }
+}
+
+// Fixed-order FP64 fold of `nparts` records of NQ doubles (max for the first
+// NMAX values, sums for the rest) by one block of kFoldThreads; the total
+// lands in s[].  Thread (q, g) folds value q over the g-th contiguous range of
+// records in record order (neighbouring q read neighbouring doubles), then
+// thread q folds the ranges in order.  The loop is bound by the latency of its
+// loads and FP64 additions, so the ranges are as many as the block holds.
+constexpr int kFoldThreads = 1024;
+template <int NQ>
+constexpr int kFoldGroups = kFoldThreads / NQ;
+template <int NQ, int NMAX>
+__device__ __forceinline__ void fold_records(const double* __restrict__ records, long long nparts, double* s,
+                                             double (*part)[NQ]) {
+  constexpr int NG = kFoldGroups<NQ>;
+  const int t = threadIdx.x;
+  if (t < NG * NQ) {
+    const int q = t % NQ, g = t / NQ;
+    const long long per = (nparts + NG - 1) / NG;
+    const long long b0 = (long long)g * per;
+    const long long b1 = (b0 + per < nparts) ? b0 + per : nparts;
+    double v = 0.0;
+#pragma unroll 8
+    for (long long b = b0; b < b1; ++b) {
+      const double x = records[b * NQ + q];
+      v = (q < NMAX) ? fmax(v, x) : v + x;
+    }
+    part[g][q] = v;
+  }
+  __syncthreads();
+  if (t < NQ) {
+    double v = part[0][t];
+#pragma unroll
+    for (int g = 1; g < NG; ++g) v = (t < NMAX) ? fmax(v, part[g][t]) : v + part[g][t];
+    s[t] = v;
+  }
+  __syncthreads();
+}
+
+// The error reduction of a single cell, by the blocks of pass A themselves: the
+// last block of each group of kTailGroup to finish folds the group's records,
+// the last group's block folds those and forms the error measure (a launch of
+// its own took 15 us: one SM's FP64 pipe, two lanes wide, had all 304 records
+// to add).  Records are folded in index order, so the result does not depend
+// on which blocks come last.
+// loop: decide the fixed-point loop on the device (Algorithm 2's while test)
+// for a launch inside a conditional WHILE node: out[6] counts the iterations
+// of the loop, which continues while no failure is recorded, err is finite,
+// err <= div_limit, err > tol, fewer than max_iter iterations ran and
+// (stag > 0) the stagnation watch (stall_step with window stag) has not
+// tripped: out[7], out[8] hold the last low and its iteration, out[10] the
+// longest gap between lows, out[9] = 1 records a stop by the watch.
+constexpr int kTailGroup = 16;
+template <class R>
+__device__ void finish_blocks(const CellDev<R>& c, double* partials, const double* acc, const ErrTail& tail) {
+  constexpr int NQ = kErrPartials, SPLIT = 2;
+  __shared__ double part[SPLIT][NQ], s[NQ];
+  __shared__ FinishScratch fin;
+  __shared__ int last;
+  const int t = threadIdx.x, grid = (int)gridDim.x, group = (int)blockIdx.x / kTailGroup;
+  const int groups = (grid + kTailGroup - 1) / kTailGroup;
+  double* records = partials + (long long)kTailRecords * NQ;  // the blocks', after the groups'
+  // true in every thread of the block that finished last of `of`
+  auto arrive = [&](unsigned* counter, int of) {
+    __threadfence();
+    __syncthreads();
+    if (t == 0) {
+      last = atomicAdd(counter, 1u) == (unsigned)(of - 1);
+      if (last) *counter = 0u;  // for the next launch
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last != 0;
+  };
+  // folds n records at r into s (max for the first four values, sums else)
+  auto fold = [&](const double* r, int n) {
+    const int q = t % NQ, g = t / NQ, per = (n + SPLIT - 1) / SPLIT;
+    if (g < SPLIT) {
+      double v = 0.0;
+#pragma unroll 8
+      for (int b = g * per; b < min(n, (g + 1) * per); ++b) {
+        const double x = __ldcg(r + (long long)b * NQ + q);
+        v = (q < 4) ? fmax(v, x) : v + x;
+      }
+      part[g][q] = v;
+    }
+    __syncthreads();
+    if (t < NQ) s[t] = (t < 4) ? fmax(part[0][t], part[1][t]) : part[0][t] + part[1][t];
+    __syncthreads();
+  };
+  for (int i = t; i < NQ; i += blockDim.x) records[(long long)blockIdx.x * NQ + i] = acc[i];
+  const int size = min(kTailGroup, grid - group * kTailGroup);
+  if (!arrive(tail.counters + group, size)) return;
+  fold(records + (long long)group * kTailGroup * NQ, size);
+  if (t < NQ) partials[group * NQ + t] = s[t];
+  if (!arrive(tail.counters + kTailRecords, groups)) return;
+  fold(partials, groups);
+  if (t < 32) finish_err<R>(c, s, tail.err_kind, tail.out, fin);
+  if (t == 0 && tail.loop) {
+    double* out = tail.out;
+    const int it = (int)out[6] + 1;
+    out[6] = (double)it;
+    const double err = out[0];
+    bool go = out[5] == 0.0 && isfinite(err) && err <= tail.div_limit && err > tail.tol && it < tail.max_iter;
+    if (go && tail.stag > 0) {
+      double ref_err = out[7];
+      int it_ref = (int)out[8], gap = (int)out[10];
+      if (stall_step(err, it, tail.stag, tail.adapt != 0, ref_err, it_ref, gap)) {
+        go = false;
+        out[9] = 1.0;
+      }
+      out[7] = ref_err;
+      out[8] = (double)it_ref;
+      out[10] = (double)gap;
+    }
+    cudaGraphSetConditional(tail.handle, go ? 1u : 0u);
+  }
+}
+
 // Pass A over a cell (single: per-block error totals in `partials`) or over
 // the entries of a multi-cell launch (per-item partials in each cell's ipart).
 template <class R, int MODE, bool MULTI>
 __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 ? 2 : 1))
     k_pass_a(CellDev<R> c0, Work<R> w, double* partials, const R* fin_tau, const R* fin_mu,
-             R* fout_e, R* fout_g) {
+             R* fout_e, R* fout_g, ErrTail tail) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CellDev<R> cs;
   __shared__ double itm[kErrPartials];
@@ -1046,172 +1238,9 @@ __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 ? 2 : 1))
     }
     __syncthreads();
     flag_timeout(status);
-    return;
   }
-  if (MODE == kIter && !MULTI) {
-    for (int i = threadIdx.x; i < kErrPartials; i += blockDim.x)
-      partials[(long long)blockIdx.x * kErrPartials + i] = acc[i];
-  }
-}
-
-// ------------------------------------------------------------------ iteration error
-// eq. err with eq. err_local (max) or eq. err_average (mean).  Denominators
-// ||<a>|| are floored by their dimensional partner through the voxel size h
-// (den_e >= h |<gamma>|, den_gamma >= |<e>| / h, den_t >= |<m>| / h,
-// den_m >= h |<t>|), since ||<gamma>|| = 0 whenever the mean curvature is zero,
-// each ||<a>|| taken as the larger of its value now and the largest of the
-// converged increments so far (a cyclic load passes through zero means).
-// out[0] = err, out[1..4] = err_e, err_t, err_gamma, err_m, out[5] = status.
-// Run by warp 0 of the block, one lane per component, then one per field (the
-// chip's FP64 pipe is narrow and its latency long: with the fold below, an
-// iteration's reduction takes 18 us between events on a 64^3 cell where one
-// thread's took 26); out[0..5] are written by lanes 0..3.
-struct FinishScratch {
-  double mean[18], dev[18], stress[18], norm[4], ratio[4];
-};
-template <class R>
-__device__ __forceinline__ void finish_err(const CellDev<R>& c, const double* s, int err_kind, double* out,
-                                           FinishScratch& w) {
-  const int lane = threadIdx.x;
-  const double iv = c.inv_nvox;
-  const int lev = lane < 9 ? 0 : 1, i = lane - 9 * lev;  // lanes 0..17: component i of the macro / micro level
-  if (lane < 18) {
-    const double mean = s[8 + lane] * iv;
-    w.mean[lane] = mean;
-    w.dev[lane] = mean - (double)(lev == 0 ? c.E[i] : c.G[i]);
-  }
-  __syncwarp();
-  // The transformed polarization was tau - tau_c = (t - T_c) - A0 (e - E) (T_c =
-  // c.tmean as read by pass A), so <t> = <tau - tau_c> + T_c + A0 (<e> - E) and
-  // likewise <m>; <t>, <m> then become the constants of the next iteration.
-  // In the increment form it was (t - t_prev) - A0 (e - e_prev), so the same
-  // formula holds with T_c = <t_prev> (the unrounded last mean) and
-  // <e_prev> = E.
-  if (lane < 18) {
-    const int k = i / 3, l = i - 3 * k, j = 3 * l + k;
-    const double* x = w.dev + 9 * lev;
-    const double a = lev == 0 ? (double)c.ref.mu + (double)c.ref.kap : (double)c.ref.beta;
-    const double b = lev == 0 ? (double)c.ref.mu - (double)c.ref.kap : (double)c.ref.gamma;
-    const double d = lev == 0 ? (double)c.ref.lam : (double)c.ref.alpha;
-    const double tr = x[0] + x[4] + x[8];
-    const double tc = c.delta_out ? c.tmean[lane] : (double)(R)c.tmean[lane];
-    const double m = s[26 + lane] * iv + tc + a * x[i] + b * x[j] + (k == l ? d * tr : 0.0);
-    w.stress[lane] = m;
-    c.tmean[lane] = m;
-  }
-  __syncwarp();
-  // fields in the order e, t, gamma, m; magnitudes: the means now or, if
-  // larger, the largest of the converged increments so far (a cyclic load
-  // passing through a zero mean)
-  if (lane < 4) {
-    const double* v = ((lane & 1) ? w.stress : w.mean) + 9 * (lane >> 1);
-    double n = 0.0;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) n += v[q] * v[q];
-    w.norm[lane] = fmax(sqrt(n), c.tmean[18 + lane]);
-  }
-  __syncwarp();
-  if (lane < 4) {
-    const double h = c.h;
-    const double other = w.norm[lane ^ 2];  // the dimensional partner: e - gamma, t - m
-    const double den = fmax(w.norm[lane], (lane == 0 || lane == 3) ? h * other : other / h);
-    const double num = (err_kind == 0) ? s[lane] : s[4 + lane] * iv;
-    const double ea = den == 0.0 ? (num == 0.0 ? 0.0 : INFINITY) : num / den;
-    w.ratio[lane] = ea;
-    out[1 + lane] = ea;
-  }
-  __syncwarp();
-  if (lane == 0) {
-    double err = 0.0;
-    for (int a = 0; a < 4; ++a)
-      if (!(w.ratio[a] <= err)) err = w.ratio[a];  // propagates NaN
-    out[0] = err;
-    out[5] = c.status ? (double)(*c.status) : 0.0;
-  }
-}
-
-// Fixed-order FP64 fold of `nparts` records of NQ doubles (max for the first
-// NMAX values, sums for the rest) by one block of kFoldThreads; the total
-// lands in s[].  Thread (q, g) folds value q over the g-th contiguous range of
-// records in record order (neighbouring q read neighbouring doubles), then
-// thread q folds the ranges in order.  The loop is bound by the latency of its
-// loads and FP64 additions, so the ranges are as many as the block holds.
-constexpr int kFoldThreads = 1024;
-template <int NQ>
-constexpr int kFoldGroups = kFoldThreads / NQ;
-template <int NQ, int NMAX>
-__device__ __forceinline__ void fold_records(const double* __restrict__ records, long long nparts, double* s,
-                                             double (*part)[NQ]) {
-  constexpr int NG = kFoldGroups<NQ>;
-  const int t = threadIdx.x;
-  if (t < NG * NQ) {
-    const int q = t % NQ, g = t / NQ;
-    const long long per = (nparts + NG - 1) / NG;
-    const long long b0 = (long long)g * per;
-    const long long b1 = (b0 + per < nparts) ? b0 + per : nparts;
-    double v = 0.0;
-#pragma unroll 8
-    for (long long b = b0; b < b1; ++b) {
-      const double x = records[b * NQ + q];
-      v = (q < NMAX) ? fmax(v, x) : v + x;
-    }
-    part[g][q] = v;
-  }
-  __syncthreads();
-  if (t < NQ) {
-    double v = part[0][t];
-#pragma unroll
-    for (int g = 1; g < NG; ++g) v = (t < NMAX) ? fmax(v, part[g][t]) : v + part[g][t];
-    s[t] = v;
-  }
-  __syncthreads();
-}
-
-template <class R>
-__global__ void __launch_bounds__(kFoldThreads) k_reduce_err(CellDev<R> c, const double* partials, int nparts,
-                                                             int err_kind, double* out) {
-  __shared__ double s[kErrPartials];
-  __shared__ double part[kFoldGroups<kErrPartials>][kErrPartials];
-  __shared__ FinishScratch fin;
-  fold_records<kErrPartials, 4>(partials, nparts, s, part);
-  if (threadIdx.x < 32) finish_err<R>(c, s, err_kind, out, fin);
-}
-
-// The same reduction, deciding the fixed-point loop on the device (Algorithm 2's
-// while test) for a launch inside a conditional WHILE node: out[6] counts the
-// iterations of the loop; the loop continues while no failure is recorded,
-// err is finite, err <= div_limit, err > tol, fewer than max_iter iterations
-// ran and (stag > 0) the stagnation watch (stall_step with window stag) has
-// not tripped: out[7], out[8] hold the last low and its iteration, out[10]
-// the longest gap between lows, out[9] = 1 records a stop by the watch.
-template <class R>
-__global__ void __launch_bounds__(kFoldThreads) k_reduce_err_loop(CellDev<R> c, const double* partials, int nparts,
-                                                                  int err_kind, double* out, double tol,
-                                                                  int max_iter, double div_limit, int stag,
-                                                                  int adapt, cudaGraphConditionalHandle handle) {
-  __shared__ double s[kErrPartials];
-  __shared__ double part[kFoldGroups<kErrPartials>][kErrPartials];
-  __shared__ FinishScratch fin;
-  fold_records<kErrPartials, 4>(partials, nparts, s, part);
-  if (threadIdx.x < 32) finish_err<R>(c, s, err_kind, out, fin);
-  if (threadIdx.x == 0) {
-    const int it = (int)out[6] + 1;
-    out[6] = (double)it;
-    const double err = out[0];
-    bool go = out[5] == 0.0 && isfinite(err) && err <= div_limit && err > tol && it < max_iter;
-    if (go && stag > 0) {
-      double ref_err = out[7];
-      int it_ref = (int)out[8], gap = (int)out[10];
-      if (stall_step(err, it, stag, adapt != 0, ref_err, it_ref, gap)) {
-        go = false;
-        out[9] = 1.0;
-      }
-      out[7] = ref_err;
-      out[8] = (double)it_ref;
-      out[10] = (double)gap;
-    }
-    cudaGraphSetConditional(handle, go ? 1u : 0u);
-  }
+  // (a failed block still counts as finished: the last one reports the status)
+  if constexpr (MODE == kIter && !MULTI) finish_blocks<R>(c0, partials, acc, tail);
 }
 
 // Algorithm 2's loop test for one batched cell after an iteration whose error
@@ -1706,40 +1735,15 @@ cudaError_t launch_green_z(const LaunchCfg& L, const CellDev<R>& c, cudaStream_t
 }
 
 template <class R>
-cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* partials,
+cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* partials, const ErrTail& tail,
                                cudaStream_t st) {
   cudaError_t e = set_smem_attrs<R>();
   if (e != cudaSuccess) return e;
+  ErrTail t = tail;
+  t.counters = reinterpret_cast<unsigned*>(partials + (size_t)(kTailRecords + L.grid_max) * kErrPartials);
   k_pass_a<R, kIter, false><<<L.grid_a, L.threads_a, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
-      c, Work<R>{}, partials, nullptr, nullptr, nullptr, nullptr);
+      c, Work<R>{}, partials, nullptr, nullptr, nullptr, nullptr, t);
   return cudaGetLastError();
-}
-
-template <class R>
-cudaError_t launch_reduce_err(const LaunchCfg& L, const CellDev<R>& c, const double* partials,
-                              int err_kind, double* err_out, cudaStream_t st) {
-  k_reduce_err<R><<<1, kFoldThreads, 0, st>>>(c, partials, L.grid_a, err_kind, err_out);
-  return cudaGetLastError();
-}
-
-template <class R>
-cudaError_t launch_reduce_err_loop(const LaunchCfg& L, const CellDev<R>& c, const double* partials, int err_kind,
-                                   double* err_out, double tol, int max_iter, double div_limit, int stag,
-                                   int adapt, cudaGraphConditionalHandle handle, cudaStream_t st) {
-  k_reduce_err_loop<R><<<1, kFoldThreads, 0, st>>>(c, partials, L.grid_a, err_kind, err_out, tol, max_iter, div_limit,
-                                          stag, adapt, handle);
-  return cudaGetLastError();
-}
-
-template <class R>
-cudaError_t launch_iteration(const LaunchCfg& L, const CellDev<R>& c, double* partials,
-                             double* err_out, int err_kind, cudaStream_t st) {
-  cudaError_t e;
-  if ((e = launch_fft_y<R>(L, c, -1, st)) != cudaSuccess) return e;
-  if ((e = launch_green_z<R>(L, c, st)) != cudaSuccess) return e;
-  if ((e = launch_fft_y<R>(L, c, +1, st)) != cudaSuccess) return e;
-  if ((e = launch_pass_a_iter<R>(L, c, partials, st)) != cudaSuccess) return e;
-  return launch_reduce_err<R>(L, c, partials, err_kind, err_out, st);
 }
 
 template <class R>
@@ -1748,7 +1752,7 @@ cudaError_t launch_start(const LaunchCfg& L, const CellDev<R>& c, int first, cud
   if (e != cudaSuccess) return e;
   if (first) k_init<R, false><<<L.grid_v, 256, 0, st>>>(c, Work<R>{});
   k_pass_a<R, kStart, false><<<L.grid_a, L.threads_a, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
-      c, Work<R>{}, nullptr, nullptr, nullptr, nullptr, nullptr);
+      c, Work<R>{}, nullptr, nullptr, nullptr, nullptr, nullptr, ErrTail{});
   return cudaGetLastError();
 }
 
@@ -1770,7 +1774,7 @@ cudaError_t launch_multi_iteration(const MultiCfg<R>& m, cudaStream_t st) {
   if (m.items_y > 0 && (e = launch_line_multi<R, kYInverse>(m.wy, m.grid_y, m.smem_y, st)) != cudaSuccess) return e;
   if (m.items_a > 0)
     k_pass_a<R, kIter, true><<<m.grid_a, kThreads, m.smem_a, st>>>(CellDev<R>{}, m.wa, nullptr, nullptr,
-                                                                    nullptr, nullptr, nullptr);
+                                                                    nullptr, nullptr, nullptr, ErrTail{});
   if (m.wa.n_act > 0) k_reduce_err_multi<R><<<m.wa.n_act, kFoldThreads, 0, st>>>(m.wa);
   return cudaGetLastError();
 }
@@ -1782,7 +1786,7 @@ cudaError_t launch_multi_start(const MultiCfg<R>& m, cudaStream_t st) {
   if (m.items_v0 > 0) k_init<R, true><<<m.grid_v0, 256, 0, st>>>(CellDev<R>{}, m.wv0);
   if (m.items_s > 0)
     k_pass_a<R, kStart, true><<<m.grid_s, kThreads, m.smem_a, st>>>(CellDev<R>{}, m.ws, nullptr, nullptr,
-                                                                     nullptr, nullptr, nullptr);
+                                                                     nullptr, nullptr, nullptr, ErrTail{});
   return cudaGetLastError();
 }
 
@@ -1822,7 +1826,7 @@ cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R*
   cudaError_t e = set_smem_attrs<R>();
   if (e != cudaSuccess) return e;
   const size_t sa = smem_pass_a<R>(c.n1, c.rows_a);
-  k_pass_a<R, kXFwd, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, tau, mu, nullptr, nullptr);
+  k_pass_a<R, kXFwd, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, tau, mu, nullptr, nullptr, ErrTail{});
   bool fused = false;
   if constexpr (sizeof(R) == 4) {
     if (ctl) {
@@ -1835,7 +1839,7 @@ cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R*
     if ((e = launch_green_z<R>(L, c, st)) != cudaSuccess) return e;
     if ((e = launch_fft_y<R>(L, c, +1, st)) != cudaSuccess) return e;
   }
-  k_pass_a<R, kXInv, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, nullptr, nullptr, e_out, g_out);
+  k_pass_a<R, kXInv, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, nullptr, nullptr, e_out, g_out, ErrTail{});
   return cudaGetLastError();
 }
 
@@ -1917,6 +1921,7 @@ LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted, bool sh
   L.threads_a = !shared && (long long)rows * c.n1 <= 128 && (sizeof(R) == 4 || 2 * smem_a <= kSmemOptin) ? 128 : kThreads;
   L.grid_a = std::min(grid_for<R>((const void*)k_pass_a<R, kIter, false>, L.threads_a, smem_a, items, nsm),
                       kPassABlocks * nsm);
+  L.grid_max = kPassABlocks * nsm;
   // Columns per y / z tile: about 256 (FP32) or 128 (FP64) points for cells
   // launched together.  A cell alone takes, in FP64, fewer where that would
   // not give every SM two tiles (16^3: the three passes took 106 us in 8 tiles
@@ -1966,14 +1971,7 @@ bool sizes_fit(int n1, int n2, int n3) {
 #define MP_INSTANTIATE(R)                                                                            \
   template cudaError_t launch_fft_y<R>(const LaunchCfg&, const CellDev<R>&, int, cudaStream_t);       \
   template cudaError_t launch_green_z<R>(const LaunchCfg&, const CellDev<R>&, cudaStream_t);          \
-  template cudaError_t launch_pass_a_iter<R>(const LaunchCfg&, const CellDev<R>&, double*, cudaStream_t); \
-  template cudaError_t launch_reduce_err_loop<R>(const LaunchCfg&, const CellDev<R>&, const double*, int, \
-                                                 double*, double, int, double, int, int,             \
-                                                 cudaGraphConditionalHandle, cudaStream_t);          \
-  template cudaError_t launch_reduce_err<R>(const LaunchCfg&, const CellDev<R>&, const double*, int,  \
-                                            double*, cudaStream_t);                                  \
-  template cudaError_t launch_iteration<R>(const LaunchCfg&, const CellDev<R>&, double*, double*, int, \
-                                           cudaStream_t);                                            \
+  template cudaError_t launch_pass_a_iter<R>(const LaunchCfg&, const CellDev<R>&, double*, const ErrTail&, cudaStream_t); \
   template cudaError_t launch_start<R>(const LaunchCfg&, const CellDev<R>&, int, cudaStream_t);       \
   template cudaError_t launch_commit<R>(const LaunchCfg&, const CellDev<R>&, double*, double*,        \
                                         cudaStream_t);                                               \

@@ -11,6 +11,7 @@ struct LaunchCfg {
   long long items_a = 1;
   int threads_a = 256;  // threads of a pass-A block
   int grid_a = 1;  // pass-A grid (persistent, one error partial per block)
+  int grid_max = 1;  // the largest grid_a of any configuration on this device
   int cols_y = 1, cols_z = 1;  // columns per tile of the y / z passes
   int grid_y = 1;
   int grid_z = 1;
@@ -66,26 +67,28 @@ template <class R>
 cudaError_t launch_fft_y(const LaunchCfg& L, const CellDev<R>& c, int dir, cudaStream_t st);
 template <class R>
 cudaError_t launch_green_z(const LaunchCfg& L, const CellDev<R>& c, cudaStream_t st);
+// What pass A's last block does with the iteration's error: the error row
+// `out` (err, the four per-field errors, status) and, with `loop`, the
+// decision of a device-run loop for `handle` (a conditional WHILE node's) in
+// out[6..10]: loop iterations, last low, its iteration, stopped by the watch,
+// longest gap between lows (out[6..9] zeroed before the loop).
+struct ErrTail {
+  unsigned* counters;  // set by the launcher (in the partials buffer)
+  double* out;
+  int err_kind, loop;
+  double tol, div_limit;
+  int max_iter, stag, adapt;
+  cudaGraphConditionalHandle handle;
+};
+// The partials buffer of a cell: group records, one record per block, arrival
+// counters (zero before the first launch; every launch leaves them zero).
+constexpr int kTailRecords = 64;
+inline size_t partials_bytes(int nsm) {
+  return sizeof(double) * kErrPartials * (size_t)(kTailRecords + kPassABlocks * nsm) + sizeof(unsigned) * (kTailRecords + 1);
+}
 template <class R>
-cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* partials, cudaStream_t st);
-template <class R>
-cudaError_t launch_reduce_err(const LaunchCfg& L, const CellDev<R>& c, const double* partials,
-                              int err_kind, double* err_out, cudaStream_t st);
-// The error reduction of a loop decided on the device: additionally counts
-// the iteration in err_out[6] (zeroed before the loop) and sets `handle` (a
-// conditional WHILE node's) to continue while err > tol, err finite and
-// <= div_limit, no failure recorded, fewer than max_iter iterations ran and
-// (stag > 0) the stagnation watch (stall_step, window stag, widening when
-// adapt) has not tripped (err_out[6..10]: loop iterations, last low, its
-// iteration, stopped by the watch, longest gap between lows).
-template <class R>
-cudaError_t launch_reduce_err_loop(const LaunchCfg& L, const CellDev<R>& c, const double* partials, int err_kind,
-                                   double* err_out, double tol, int max_iter, double div_limit, int stag,
-                                   int adapt, cudaGraphConditionalHandle handle, cudaStream_t st);
-// One fixed-point iteration; writes err and the four per-field errors to err_out[0..4].
-template <class R>
-cudaError_t launch_iteration(const LaunchCfg& L, const CellDev<R>& c, double* partials,
-                             double* err_out, int err_kind, cudaStream_t st);
+cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* partials, const ErrTail& tail,
+                               cudaStream_t st);
 // Start of a load increment: (first ? zero state + e = E : predictor already in place),
 // Algorithm 1 at the predictor, polarizations, forward x transform.
 template <class R>

@@ -358,9 +358,12 @@ template <class R>
 __host__ __device__ constexpr int line_threads(int pass) {
   return pass < kZReduced ? LineCfg<R>::y_threads : LineCfg<R>::z_threads;
 }
+// (FP64 y passes of small radices fit four blocks' registers without spills.)
 template <class R>
-__host__ __device__ constexpr int line_blocks(int pass) {
-  return pass < kZReduced ? LineCfg<R>::y_blocks : pass == kZReduced ? LineCfg<R>::z_blocks : 2;
+__host__ __device__ constexpr int line_blocks(int pass, int n) {
+  return pass < kZReduced ? LineCfg<R>::y_blocks + (sizeof(R) == 8 && line_plan(n).r0 <= 9 ? 1 : 0)
+         : pass == kZReduced ? LineCfg<R>::z_blocks
+                             : 2;
 }
 
 template <class R, int PASS, int N>
@@ -388,13 +391,13 @@ __device__ __forceinline__ void line_tile(const CellDev<R>& c, long long tile, c
 
 // One cell, one length.
 template <class R, int PASS, int N>
-__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS)) k_fft_y(CellDev<R> c) {
+__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS, N)) k_fft_y(CellDev<R> c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   for (long long t = blockIdx.x; t < tiles_y(c); t += gridDim.x)
     line_tile<R, PASS, N>(c, t, reinterpret_cast<cpx<R>*>(smem_raw), t == (long long)blockIdx.x);
 }
 template <class R, int PASS, int N>
-__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS)) k_green_z(CellDev<R> c) {
+__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS, N)) k_green_z(CellDev<R> c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   for (long long t = blockIdx.x; t < tiles_z(c); t += gridDim.x)
     line_tile<R, PASS, N>(c, t, reinterpret_cast<cpx<R>*>(smem_raw), t == (long long)blockIdx.x);
