@@ -11,6 +11,8 @@
 // tau = t - A0 e, mu = m - B0 gamma, forward x transform.
 #include "mp_kernels.cuh"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -922,31 +924,39 @@ __device__ __forceinline__ bool pass_a_item(const CellDev<R>& c, long long item,
       }
     }
     // Row sums.  With the unnormalised inverse along x, sum_x e~ = N1 X_in[0],
-    // so sum_x e = N1 (E + X_in[0]); the forward DC is sum_x tau.
+    // so sum_x e = N1 (E + X_in[0]); the forward DC is sum_x tau.  Thread q + 36 k
+    // sums value q over rows k, k + P, ... (P groups of 36 threads): the FP64
+    // pipe takes a warp's instruction in 17 cycles however few lanes it has, and
+    // 36 threads over all 16 rows of a 16^3 item kept it busy for 3200.
+    double* csum = reinterpret_cast<double*>(smem_raw + L.carry_off + kThreads * (4 * sizeof(R) + 4 * sizeof(double)));
+    const int P = (int)blockDim.x / 36, part = (int)threadIdx.x / 36, q = (int)threadIdx.x - 36 * part;
     double rsum = 0.0;
-    const int q = threadIdx.x - 32;
-    if (q >= 0 && q < 36) {
+    if (part < P && part < nr) {
       if (q < 18) {
         const double mean = (double)((q < 9) ? c.E[q] : c.G[q - 9]);
-        for (int rr = 0; rr < nr; ++rr) rsum += (double)N1 * (mean + (double)dcin[q * rows + rr]);
+        for (int rr = part; rr < nr; rr += P) rsum += (double)dcin[q * rows + rr];
+        rsum = (double)N1 * ((double)((nr - part + P - 1) / P) * mean + rsum);
       } else {
-        for (int rr = 0; rr < nr; ++rr) rsum += (double)X[rr * M * 18 + (q - 18)].x;
+        for (int rr = part; rr < nr; rr += P) rsum += (double)X[rr * M * 18 + (q - 18)].x;
       }
-      if constexpr (!MULTI)
-        reinterpret_cast<double*>(smem_raw + L.carry_off + kThreads * (4 * sizeof(R) + 4 * sizeof(double)))[threadIdx.x] += rsum;
     }
+    if constexpr (!MULTI) csum[threadIdx.x] += rsum;
+    else csum[threadIdx.x] = rsum;
     if constexpr (MULTI) {
       __syncthreads();
       const int nwarp = blockDim.x >> 5;
-      if (threadIdx.x < 8) {
-        double a = red[threadIdx.x];
+      if (threadIdx.x < 36) {
+        double v = csum[threadIdx.x];
+        for (int k = 1; k < P && k < nr; ++k) v += csum[threadIdx.x + 36 * k];
+        itm[8 + threadIdx.x] = v;
+      } else if (threadIdx.x >= 64 && threadIdx.x < 72) {
+        const int w0 = (int)threadIdx.x - 64;
+        double v = red[w0];
         for (int w = 1; w < nwarp; ++w) {
-          const double vv = red[w * 8 + threadIdx.x];
-          a = (threadIdx.x < 4) ? fmax(a, vv) : a + vv;
+          const double vv = red[w * 8 + w0];
+          v = (w0 < 4) ? fmax(v, vv) : v + vv;
         }
-        itm[threadIdx.x] = a;
-      } else if (q >= 0 && q < 36) {
-        itm[8 + q] = rsum;
+        itm[w0] = v;
       }
     }
   }
@@ -1036,7 +1046,7 @@ __device__ __forceinline__ void finish_err(const CellDev<R>& c, const double* s,
 // records in record order (neighbouring q read neighbouring doubles), then
 // thread q folds the ranges in order.  The loop is bound by the latency of its
 // loads and FP64 additions, so the ranges are as many as the block holds.
-constexpr int kFoldThreads = 1024;
+constexpr int kFoldThreads = 512;
 template <int NQ>
 constexpr int kFoldGroups = kFoldThreads / NQ;
 template <int NQ, int NMAX>
@@ -1224,9 +1234,13 @@ __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 ? 2 : 1))
       }
       acc[threadIdx.x] = a;
     }
-    const int q = threadIdx.x - 32;
-    if (q >= 0 && q < 36)
-      acc[8 + q] = reinterpret_cast<const double*>(smem_raw + SL.carry_off + kThreads * (4 * sizeof(R) + 4 * sizeof(double)))[threadIdx.x];
+    if (threadIdx.x < 36) {
+      const double* csum = reinterpret_cast<const double*>(smem_raw + SL.carry_off +
+                                                           kThreads * (4 * sizeof(R) + 4 * sizeof(double)));
+      double v = csum[threadIdx.x];
+      for (int k = 1; k < (int)blockDim.x / 36; ++k) v += csum[threadIdx.x + 36 * k];
+      acc[8 + threadIdx.x] = v;
+    }
     __syncthreads();
   }
   if (threadIdx.x == 0) bulk_wait_all();
@@ -1271,19 +1285,40 @@ __device__ void round_decide(RoundCtl& rc, const double* e) {
   rc.stop = stop ? 1 : 0;
 }
 
-// One block per entry: the cell's per-item partials.
+// One cluster of kFoldCluster blocks per entry: each folds a quarter of the
+// cell's per-item records on its own SM's FP64 pipe (one block took 24 us for
+// the 461 records of a 48^3 cell), the first takes the others' totals from
+// their shared memory, in rank order.
+constexpr int kFoldCluster = 4;
 template <class R>
-__global__ void __launch_bounds__(kFoldThreads) k_reduce_err_multi(Work<R> w) {
+__global__ void __cluster_dims__(kFoldCluster, 1, 1) __launch_bounds__(kFoldThreads) k_reduce_err_multi(Work<R> w) {
+  namespace cg = cooperative_groups;
   __shared__ double s[kErrPartials];
   __shared__ double part[kFoldGroups<kErrPartials>][kErrPartials];
   __shared__ FinishScratch fin;
   __shared__ CellDev<R> cs;
-  load_cell(cs, w.cells + w.act[blockIdx.x]);
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  load_cell(cs, w.cells + w.act[blockIdx.x / kFoldCluster]);
   __syncthreads();
   RoundCtl* rc = cs.rctl;
-  if (rc != nullptr && __ldcg(&rc->stop) != 0) return;  // uniform: one flag per block
-  fold_records<kErrPartials, 4>(cs.ipart, cs.items_a, s, part);
-  if (threadIdx.x < 32) {
+  // (uniform over the cluster: the flag only changes at the end of this kernel,
+  // after the cluster's last barrier)
+  if (rc != nullptr && __ldcg(&rc->stop) != 0) return;
+  const long long per = (cs.items_a + kFoldCluster - 1) / kFoldCluster, b0 = rank * per;
+  const long long n = cs.items_a - b0 < per ? cs.items_a - b0 : per;
+  fold_records<kErrPartials, 4>(cs.ipart + b0 * kErrPartials, n > 0 ? n : 0, s, part);
+  cluster.sync();
+  if (rank == 0 && threadIdx.x < kErrPartials) {
+    double v = s[threadIdx.x];
+    for (int k = 1; k < kFoldCluster; ++k) {
+      const double x = cluster.map_shared_rank(s, k)[threadIdx.x];
+      v = (threadIdx.x < 4) ? fmax(v, x) : v + x;
+    }
+    s[threadIdx.x] = v;
+  }
+  cluster.sync();  // the others' shared memory lives until it has been read
+  if (rank == 0 && threadIdx.x < 32) {
     double* out = rc != nullptr ? rc->rows + 8 * rc->rounds : cs.err_out;
     finish_err<R>(cs, s, cs.err_kind, out, fin);
     __syncwarp();
@@ -1301,20 +1336,20 @@ __device__ __forceinline__ void init_chunk(const CellDev<R>& c, long long chunk)
   R* pv = c.prev + v * 20;
   R* hv = c.hist + v * 20;
   R* el = c.elast + v * 18;
+  // in 16- / 8-byte pieces (value by value a 256^3 FP32 cell took 4.9 ms)
+  R rec[20];
 #pragma unroll
   for (int q = 0; q < 9; ++q) {
-    pv[q] = c.E[q];
-    pv[9 + q] = c.G[q];
+    rec[q] = c.E[q];
+    rec[9 + q] = c.G[q];
   }
-  pv[18] = R(1);
-  pv[19] = R(1);
+  rec[18] = rec[19] = R(1);
+  store_rec(pv, rec);
 #pragma unroll
-  for (int q = 0; q < 18; ++q) {
-    hv[q] = R(0);
-    el[q] = R(0);
-  }
-  hv[18] = (R)c.phase[v];  // phase id travels with the history record
-  hv[19] = R(0);
+  for (int q = 0; q < 20; ++q) rec[q] = R(0);
+  store_rec18(el, rec);
+  rec[18] = (R)c.phase[v];  // phase id travels with the history record
+  store_rec(hv, rec);
   reinterpret_cast<double2*>(c.pq)[v] = make_double2(0.0, 0.0);
 }
 
@@ -1418,18 +1453,45 @@ __device__ __forceinline__ void commit_chunk(const CellDev<R>& c, long long chun
     }
     return;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // Records per chunk: the field-type values are transposed through shared
+  // memory and summed by (value, part) threads - FP32 values in compensated
+  // pairs, folded in FP64 - and p, q by warp shuffles.  (Shuffling all 40
+  // values in FP64 cost 1600 warp additions a chunk on the FP64 pipe, 17 cycles
+  // each: the commit of a 32-cell batch took 755 us.)
+  constexpr int PITCH = 257, PARTS = 6, LEN = (256 + PARTS - 1) / PARTS;
+  R* tile = reinterpret_cast<R*>(cols);  // [kAvgPartials][PITCH]
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
 #pragma unroll
-  for (int i = 0; i < kAvgPartials; ++i) {
-    const double x = (i == 36) ? p : (i == 37) ? q : (double)val[i];
-    const double sm = shfl_sum(x);
-    if (lane == 0) red[warp][i] = sm;
+  for (int i = 0; i < kAvgPartials; ++i)
+    if (i != 36 && i != 37) tile[i * PITCH + t] = val[i];
+  const double ps = shfl_sum(p), qs = shfl_sum(q);
+  if (lane == 0) {
+    red[warp][36] = ps;
+    red[warp][37] = qs;
   }
   __syncthreads();
-  if (threadIdx.x < kAvgPartials) {
+  if (t < PARTS * kAvgPartials) {
+    const int i = t % kAvgPartials, part = t / kAvgPartials;
+    if (i != 36 && i != 37) {
+      const R* v = tile + i * PITCH;
+      const int k1 = min(256, (part + 1) * LEN);
+      double sm = 0.0;
+      if constexpr (sizeof(R) == 4) {
+        float2 acc = make_float2(0.f, 0.f);
+        for (int k = part * LEN; k < k1; ++k) two_sum_acc(acc, v[k]);
+        sm = (double)acc.x + (double)acc.y;
+      } else {
+        for (int k = part * LEN; k < k1; ++k) sm += v[k];
+      }
+      red[part][i] = sm;
+    }
+  }
+  __syncthreads();
+  if (t < kAvgPartials) {
     double sm = 0.0;
-    for (int wq = 0; wq < (bd >> 5); ++wq) sm += red[wq][threadIdx.x];
-    out40[threadIdx.x] = sm;
+    const int n = (t == 36 || t == 37) ? (bd >> 5) : PARTS;
+    for (int k = 0; k < n; ++k) sm += red[k][t];
+    out40[t] = sm;
   }
   __syncthreads();
 }
@@ -1441,7 +1503,8 @@ __device__ __forceinline__ void commit_chunk(const CellDev<R>& c, long long chun
 // per-chunk records in each cell's apart.
 template <class R, bool MULTI>
 __global__ void __launch_bounds__(256) k_commit(CellDev<R> c0, Work<R> w, double* partials) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];  // single: [kAvgPartials][256] 8-byte slots
+  // single: [kAvgPartials][256] 8-byte slots; multi: the chunk's values, [kAvgPartials][257] of R
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CellDev<R> cs;
   __shared__ double red[8][kAvgPartials];
   __shared__ double chunk_sum[kAvgPartials];
@@ -1656,6 +1719,8 @@ __global__ void __launch_bounds__(kPointThreads)
 template <class R>
 size_t smem_pass_a(int n1, int rows) { return PassASmem<R>(n1, rows).total; }
 
+template <class R>
+constexpr size_t kCommitTile = (size_t)kAvgPartials * 257 * sizeof(R);  // multi-cell commit, a chunk's values
 constexpr size_t kCommitSmem = (size_t)kAvgPartials * 256 * sizeof(double);  // single-cell commit columns
 
 // Raise the dynamic shared-memory limit of the kernels launched without a
@@ -1687,6 +1752,7 @@ static cudaError_t set_smem_attrs() {
   raise((const void*)k_pass_a<R, kIter, true>);
   raise((const void*)k_pass_a<R, kStart, true>);
   raise((const void*)k_commit<R, false>, false);
+  raise((const void*)k_commit<R, true>, false);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -1775,7 +1841,7 @@ cudaError_t launch_multi_iteration(const MultiCfg<R>& m, cudaStream_t st) {
   if (m.items_a > 0)
     k_pass_a<R, kIter, true><<<m.grid_a, kThreads, m.smem_a, st>>>(CellDev<R>{}, m.wa, nullptr, nullptr,
                                                                     nullptr, nullptr, nullptr, ErrTail{});
-  if (m.wa.n_act > 0) k_reduce_err_multi<R><<<m.wa.n_act, kFoldThreads, 0, st>>>(m.wa);
+  if (m.wa.n_act > 0) k_reduce_err_multi<R><<<m.wa.n_act * kFoldCluster, kFoldThreads, 0, st>>>(m.wa);
   return cudaGetLastError();
 }
 
@@ -1792,7 +1858,9 @@ cudaError_t launch_multi_start(const MultiCfg<R>& m, cudaStream_t st) {
 
 template <class R>
 cudaError_t launch_multi_commit(const MultiCfg<R>& m, cudaStream_t st) {
-  if (m.items_v > 0) k_commit<R, true><<<m.grid_v, 256, 0, st>>>(CellDev<R>{}, m.wv, nullptr);
+  const cudaError_t e = set_smem_attrs<R>();
+  if (e != cudaSuccess) return e;
+  if (m.items_v > 0) k_commit<R, true><<<m.grid_v, 256, kCommitTile<R>, st>>>(CellDev<R>{}, m.wv, nullptr);
   if (m.wv.n_act > 0) k_reduce_avg_multi<R><<<m.wv.n_act, kFoldThreads, 0, st>>>(m.wv);
   return cudaGetLastError();
 }

@@ -419,7 +419,7 @@ __device__ __forceinline__ void line_tile_any(const CellDev<R>& c, long long til
   }
 }
 template <class R, int PASS>
-__global__ void __launch_bounds__(line_threads<R>(PASS), 2) k_line_multi(Work<R> w) {
+__global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS, 256)) k_line_multi(Work<R> w) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CellDev<R> cs;
   for_items<R, true>(CellDev<R>{}, 0, w, cs, [&](const CellDev<R>& c, long long t, bool fresh) {
