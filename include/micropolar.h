@@ -235,7 +235,7 @@ mp_status mp_rve_config(const mp_rve* rve, int32_t* cfg, int32_t n);
 #define MP_KC_GREEN_Z 1   /* z forward + Green operator + z inverse pass                */
 #define MP_KC_FFT_Y_INV 2 /* y-direction inverse transform pass                         */
 #define MP_KC_PASS_A 3    /* x inverse, Algorithm 1, error partials, polarization, x fwd */
-#define MP_KC_REDUCE 4    /* iteration error reduction                                   */
+#define MP_KC_REDUCE 4    /* iteration error reduction (part of pass A: no launches)      */
 #define MP_KC_START 5     /* increment start: initial state, predictor pass              */
 #define MP_KC_COMMIT 6    /* commit of a converged increment and homogenized averages    */
 #define MP_KC_SPECTRAL 7  /* fused pass: y fwd, z fwd, Green operator, z inv, y inv       */

@@ -1,8 +1,7 @@
 // Transform plans of one axis (host side): the radix sequence and the twiddle
 // table W_N^k = exp(-2 pi i k / N).  Header-only, with no dependency on the
 // library context, so that every entry point (allocating or not) builds its
-// plans from the same code; the compile-time stage sequences of the kernels
-// (mp_fft.cuh, mp_kernels.cu) assume exactly these radix sequences.
+// plans from the same code.
 #pragma once
 
 #include <cmath>
@@ -14,11 +13,10 @@
 
 namespace mp {
 
-// Radix sequence of a complex transform of length m = 2^a 3^b.  Powers of two
-// take as few stages as possible, radix 16 only where it saves one (allow16;
-// the x axis, transformed inside pass A, is limited to radix 8); radix-3
-// stages come last.
-inline void radix_plan(int m, int* radix, int& nst, bool allow16) {
+// Radix sequence of the packed x axis' complex transform of length m = 2^a 3^b
+// (for the lengths without compile-time stages): powers of two in as few
+// radix-8 stages as possible, radix-3 stages last.
+inline void radix_plan(int m, int* radix, int& nst) {
   nst = 0;
   int k2 = 0;
   while (m % 2 == 0) {
@@ -30,12 +28,9 @@ inline void radix_plan(int m, int* radix, int& nst, bool allow16) {
     m /= 3;
     ++k3;
   }
-  static const int kPlan2[10][4] = {{0}, {2}, {4}, {8}, {16}, {8, 4}, {8, 8}, {16, 8}, {16, 16}, {8, 8, 8}};
-  static const int kPlan2x[10][4] = {{0}, {2}, {4}, {8}, {4, 4}, {8, 4}, {8, 8}, {8, 4, 4}, {8, 8, 4}, {8, 8, 8}};
-  static const int kLen2[10] = {0, 1, 1, 1, 1, 2, 2, 2, 2, 3};
-  static const int kLen2x[10] = {0, 1, 1, 1, 2, 2, 2, 3, 3, 3};
-  const int len = allow16 ? kLen2[k2] : kLen2x[k2];
-  for (int i = 0; i < len; ++i) radix[nst++] = allow16 ? kPlan2[k2][i] : kPlan2x[k2][i];
+  static const int kPlan2[10][3] = {{0}, {2}, {4}, {8}, {4, 4}, {8, 4}, {8, 8}, {8, 4, 4}, {8, 8, 4}, {8, 8, 8}};
+  static const int kLen2[10] = {0, 1, 1, 1, 2, 2, 2, 3, 3, 3};
+  for (int i = 0; i < kLen2[k2]; ++i) radix[nst++] = kPlan2[k2][i];
   for (int i = 0; i < k3; ++i) radix[nst++] = 3;
 }
 
@@ -48,7 +43,8 @@ void axis_plan(int n, bool packed, AxisPlan<R>& p, cpx<R>* host_tw) {
   p.n = n;
   p.m = packed ? (n > 1 ? n / 2 : 1) : n;
   p.tstride = packed ? 2 : 1;
-  radix_plan(p.m, p.radix, p.nstages, !packed);
+  p.nstages = 0;  // the y / z lines have compile-time plans (line_plan)
+  if (packed) radix_plan(p.m, p.radix, p.nstages);
   for (int k = 0; k < n; ++k) {
     const double a = 2.0 * M_PI * (double)k / (double)n;
     host_tw[k].x = (R)std::cos(a);
