@@ -35,10 +35,10 @@ __device__ __forceinline__ void dft3(cpx<R>* v) {
   const R s3 = R(0.86602540378443864676372317075294);
   cpx<R> a = v[0], t = cadd(v[1], v[2]), u = csub(v[1], v[2]);
   cpx<R> base = cmake<R>(a.x - half * t.x, a.y - half * t.y);
-  cpx<R> r = rot90<R, DIR>(cscale(u, s3));
+  const cpx<R> r = rot90<R, DIR>(u);
   v[0] = cadd(a, t);
-  v[1] = cadd(base, r);
-  v[2] = csub(base, r);
+  v[1] = cfma(r, s3, base);
+  v[2] = cfma(r, -s3, base);
 }
 
 template <class R, int DIR>
@@ -66,17 +66,17 @@ __device__ __forceinline__ void dft8(cpx<R>* v) {
   dft4<R, DIR>(o);
   const R h = R(0.70710678118654752440084436210485);
   // W_8^1 = h (1 + DIR i), W_8^2 = DIR i, W_8^3 = h (-1 + DIR i)
-  cpx<R> o1 = cmake<R>(h * (o[1].x - DIR * o[1].y), h * (o[1].y + DIR * o[1].x));
+  cpx<R> o1 = cmake<R>(o[1].x - DIR * o[1].y, o[1].y + DIR * o[1].x);
   cpx<R> o2 = rot90<R, DIR>(o[2]);
-  cpx<R> o3 = cmake<R>(h * (-o[3].x - DIR * o[3].y), h * (-o[3].y + DIR * o[3].x));
+  cpx<R> o3 = cmake<R>(-o[3].x - DIR * o[3].y, -o[3].y + DIR * o[3].x);
   v[0] = cadd(e[0], o[0]);
   v[4] = csub(e[0], o[0]);
-  v[1] = cadd(e[1], o1);
-  v[5] = csub(e[1], o1);
+  v[1] = cfma(o1, h, e[1]);
+  v[5] = cfma(o1, -h, e[1]);
   v[2] = cadd(e[2], o2);
   v[6] = csub(e[2], o2);
-  v[3] = cadd(e[3], o3);
-  v[7] = csub(e[3], o3);
+  v[3] = cfma(o3, h, e[3]);
+  v[7] = cfma(o3, -h, e[3]);
 }
 
 // 16-point DFT as 4 x 4: 4-point DFTs over n1 of x[4 n1 + n2], twiddles

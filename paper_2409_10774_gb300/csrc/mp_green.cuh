@@ -39,8 +39,8 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
     cpx<R> a = cmake<R>(R(0), R(0)), b = cmake<R>(R(0), R(0));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      a = cadd(a, cscale(v[3 * k + l], xi[k]));
-      b = cadd(b, cscale(v[9 + 3 * k + l], xi[k]));
+      a = cfma(v[3 * k + l], xi[k], a);
+      b = cfma(v[9 + 3 * k + l], xi[k], b);
     }
     f[l] = cmuli(a);
     g[l] = cmuli(b);
@@ -62,28 +62,28 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
   cpx<R> xf = cmake<R>(R(0), R(0)), xg = cmake<R>(R(0), R(0));
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    xf = cadd(xf, cscale(f[l], xi[l]));
-    xg = cadd(xg, cscale(g[l], xi[l]));
+    xf = cfma(f[l], xi[l], xf);
+    xg = cfma(g[l], xi[l], xg);
   }
   // cross products xi x g, xi x f
   cpx<R> cg[3], cf[3];
-  cg[0] = csub(cscale(g[2], x2), cscale(g[1], x3));
-  cg[1] = csub(cscale(g[0], x3), cscale(g[2], x1));
-  cg[2] = csub(cscale(g[1], x1), cscale(g[0], x2));
-  cf[0] = csub(cscale(f[2], x2), cscale(f[1], x3));
-  cf[1] = csub(cscale(f[0], x3), cscale(f[2], x1));
-  cf[2] = csub(cscale(f[1], x1), cscale(f[0], x2));
+  cg[0] = cfma(g[1], -x3, cscale(g[2], x2));
+  cg[1] = cfma(g[2], -x1, cscale(g[0], x3));
+  cg[2] = cfma(g[0], -x2, cscale(g[1], x1));
+  cf[0] = cfma(f[1], -x3, cscale(f[2], x2));
+  cf[1] = cfma(f[2], -x1, cscale(f[0], x3));
+  cf[2] = cfma(f[0], -x2, cscale(f[1], x1));
 
   cpx<R> u[3], ph[3];
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
     // P f = f - xi (xi.f)/k^2 ;  -c (xi x g) = i twok (xi x g)
-    cpx<R> Pf = csub(f[l], cscale(xf, xi[l] * ik2));
-    cpx<R> Pg = csub(g[l], cscale(xg, xi[l] * ik2));
-    cpx<R> tu = cadd(cscale(Pf, b), cmuli(cscale(cg[l], twok)));
-    cpx<R> tp = cadd(cscale(Pg, a), cmuli(cscale(cf[l], twok)));
-    u[l] = cadd(cscale(xf, xi[l] * iL_u), cscale(tu, iD));
-    ph[l] = cadd(cscale(xg, xi[l] * iL_p), cscale(tp, iD));
+    cpx<R> Pf = cfma(xf, -(xi[l] * ik2), f[l]);
+    cpx<R> Pg = cfma(xg, -(xi[l] * ik2), g[l]);
+    cpx<R> tu = cfma(Pf, b, cmuli(cscale(cg[l], twok)));
+    cpx<R> tp = cfma(Pg, a, cmuli(cscale(cf[l], twok)));
+    u[l] = cfma(tu, iD, cscale(xf, xi[l] * iL_u));
+    ph[l] = cfma(tp, iD, cscale(xg, xi[l] * iL_p));
   }
   // e^_kl = i xi_k u_l + eps_lkm phi_m ; gamma^_kl = i phi_k xi_l, scaled, each
   // component written once.
@@ -97,13 +97,12 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-      cpx<R> ev = cmuli(cscale(u[l], xi[k]));
-      if (k == 0 && l == 1) ev = csub(ev, ph[2]);
-      if (k == 1 && l == 0) ev = cadd(ev, ph[2]);
-      if (k == 0 && l == 2) ev = cadd(ev, ph[1]);
-      if (k == 2 && l == 0) ev = csub(ev, ph[1]);
-      if (k == 1 && l == 2) ev = csub(ev, ph[0]);
-      if (k == 2 && l == 1) ev = cadd(ev, ph[0]);
+      // eps_lkm phi_m, m = 3 - k - l: -phi_m for (k, l) cyclic, +phi_m else
+      const cpx<R> iu = cmuli(u[l]);
+      cpx<R> ev;
+      if (k == l) ev = cscale(iu, xi[k]);
+      else if (l == (k + 1) % 3) ev = cfma(iu, xi[k], cmake<R>(-ph[3 - k - l].x, -ph[3 - k - l].y));
+      else ev = cfma(iu, xi[k], ph[3 - k - l]);
       v[3 * k + l] = ev;
       v[9 + 3 * k + l] = cmuli(cscale(ph[k], xi[l]));
     }
@@ -141,26 +140,26 @@ __device__ __forceinline__ void green_point_reduced(const RefDev<R>& A0, R x1, R
   cpx<R> xf = cmake<R>(R(0), R(0)), xg = cmake<R>(R(0), R(0));
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    xf = cadd(xf, cscale(f[l], xi[l]));
-    xg = cadd(xg, cscale(g[l], xi[l]));
+    xf = cfma(f[l], xi[l], xf);
+    xg = cfma(g[l], xi[l], xg);
   }
   cpx<R> cg[3], cf[3];  // xi x g, xi x f
-  cg[0] = csub(cscale(g[2], x2), cscale(g[1], x3));
-  cg[1] = csub(cscale(g[0], x3), cscale(g[2], x1));
-  cg[2] = csub(cscale(g[1], x1), cscale(g[0], x2));
-  cf[0] = csub(cscale(f[2], x2), cscale(f[1], x3));
-  cf[1] = csub(cscale(f[0], x3), cscale(f[2], x1));
-  cf[2] = csub(cscale(f[1], x1), cscale(f[0], x2));
+  cg[0] = cfma(g[1], -x3, cscale(g[2], x2));
+  cg[1] = cfma(g[2], -x1, cscale(g[0], x3));
+  cg[2] = cfma(g[0], -x2, cscale(g[1], x1));
+  cf[0] = cfma(f[1], -x3, cscale(f[2], x2));
+  cf[1] = cfma(f[2], -x1, cscale(f[0], x3));
+  cf[2] = cfma(f[0], -x2, cscale(f[1], x1));
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    const cpx<R> Pf = csub(f[l], cscale(xf, xi[l] * ik2));
-    const cpx<R> Pg = csub(g[l], cscale(xg, xi[l] * ik2));
-    const cpx<R> tu = cadd(cscale(Pf, b), cmuli(cscale(cg[l], twok)));
-    const cpx<R> tp = cadd(cscale(Pg, a), cmuli(cscale(cf[l], twok)));
+    const cpx<R> Pf = cfma(xf, -(xi[l] * ik2), f[l]);
+    const cpx<R> Pg = cfma(xg, -(xi[l] * ik2), g[l]);
+    const cpx<R> tu = cfma(Pf, b, cmuli(cscale(cg[l], twok)));
+    const cpx<R> tp = cfma(Pg, a, cmuli(cscale(cf[l], twok)));
     __align__(16) cpx<R> q[4];
-    q[0] = cadd(cscale(xf, xi[l] * iL_u), cscale(tu, iD));
+    q[0] = cfma(tu, iD, cscale(xf, xi[l] * iL_u));
     q[1] = cmuli(cscale(q[0], x3));
-    q[2] = cadd(cscale(xg, xi[l] * iL_p), cscale(tp, iD));
+    q[2] = cfma(tp, iD, cscale(xg, xi[l] * iL_p));
     q[3] = cmuli(cscale(q[2], x3));
 #pragma unroll
     for (int i = 0; i < (int)sizeof(q) / 16; ++i)
