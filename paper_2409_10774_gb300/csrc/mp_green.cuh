@@ -54,10 +54,12 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
   const R ik2 = R(1) / k2;
   const R a = (A0.mu + A0.kap) * k2;
   const R b = A0.gamma * k2 + R(4) * A0.kap;
-  const R twok = R(2) * A0.kap;   // c = -i twok
   const R iD = R(1) / (k2 * ((A0.mu + A0.kap) * A0.gamma * k2 + R(4) * A0.kap * A0.mu));
-  const R iL_u = ik2 * ik2 / (A0.lam + R(2) * A0.mu);
-  const R iL_p = ik2 / ((A0.alpha + A0.beta + A0.gamma) * k2 + R(4) * A0.kap);
+  // u = f u_f + xi (xi.f) u_x + i c_i (xi x g): the projection's terms collected
+  // (three roundings a component; P f, b P f and c (xi x g) in turn took five)
+  const R u_f = b * iD, p_g = a * iD, c_i = R(2) * A0.kap * iD;
+  const R u_x = fma(-u_f, ik2, ik2 * ik2 / (A0.lam + R(2) * A0.mu));
+  const R p_x = fma(-p_g, ik2, ik2 / ((A0.alpha + A0.beta + A0.gamma) * k2 + R(4) * A0.kap));
 
   cpx<R> xf = cmake<R>(R(0), R(0)), xg = cmake<R>(R(0), R(0));
 #pragma unroll
@@ -77,13 +79,8 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
   cpx<R> u[3], ph[3];
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    // P f = f - xi (xi.f)/k^2 ;  -c (xi x g) = i twok (xi x g)
-    cpx<R> Pf = cfma(xf, -(xi[l] * ik2), f[l]);
-    cpx<R> Pg = cfma(xg, -(xi[l] * ik2), g[l]);
-    cpx<R> tu = cfma(Pf, b, cmuli(cscale(cg[l], twok)));
-    cpx<R> tp = cfma(Pg, a, cmuli(cscale(cf[l], twok)));
-    u[l] = cfma(tu, iD, cscale(xf, xi[l] * iL_u));
-    ph[l] = cfma(tp, iD, cscale(xg, xi[l] * iL_p));
+    u[l] = cfma(f[l], u_f, cfma(xf, xi[l] * u_x, cmuli(cscale(cg[l], c_i))));
+    ph[l] = cfma(g[l], p_g, cfma(xg, xi[l] * p_x, cmuli(cscale(cf[l], c_i))));
   }
   // e^_kl = i xi_k u_l + eps_lkm phi_m ; gamma^_kl = i phi_k xi_l, scaled, each
   // component written once.
@@ -111,7 +108,8 @@ __device__ __forceinline__ void green_point(const RefDev<R>& A0, R x1, R x2, R x
 
 // The same operator on the 12 reduced values of a point (mp_lines.cuh): in,
 // for l = 0..2, v[4l..4l+3] = A_l, T_l, B_l, M_l with f_l = A_l + i x3 T_l and
-// g_l = B_l + i x3 M_l; out u_l, i x3 u_l, phi_l, i x3 phi_l times `scale`.
+// g_l = B_l + i x3 M_l; out u_l, e_3l = i x3 u_l + eps_l3m phi_m, phi_l,
+// gamma_l3 = i x3 phi_l times `scale`.
 // v points to shared memory, 16-byte aligned; it moves in 16-byte pieces.
 template <class R>
 __device__ __forceinline__ void green_point_reduced(const RefDev<R>& A0, R x1, R x2, R x3, cpx<R>* v, R scale) {
@@ -133,10 +131,10 @@ __device__ __forceinline__ void green_point_reduced(const RefDev<R>& A0, R x1, R
   const R ik2 = R(1) / k2;
   const R a = (A0.mu + A0.kap) * k2;
   const R b = A0.gamma * k2 + R(4) * A0.kap;
-  const R twok = R(2) * A0.kap;  // c = -i twok
   const R iD = scale / (k2 * ((A0.mu + A0.kap) * A0.gamma * k2 + R(4) * A0.kap * A0.mu));
-  const R iL_u = scale * ik2 * ik2 / (A0.lam + R(2) * A0.mu);
-  const R iL_p = scale * ik2 / ((A0.alpha + A0.beta + A0.gamma) * k2 + R(4) * A0.kap);
+  const R u_f = b * iD, p_g = a * iD, c_i = R(2) * A0.kap * iD;
+  const R u_x = fma(-u_f, ik2, scale * ik2 * ik2 / (A0.lam + R(2) * A0.mu));
+  const R p_x = fma(-p_g, ik2, scale * ik2 / ((A0.alpha + A0.beta + A0.gamma) * k2 + R(4) * A0.kap));
   cpx<R> xf = cmake<R>(R(0), R(0)), xg = cmake<R>(R(0), R(0));
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
@@ -150,17 +148,21 @@ __device__ __forceinline__ void green_point_reduced(const RefDev<R>& A0, R x1, R
   cf[0] = cfma(f[1], -x3, cscale(f[2], x2));
   cf[1] = cfma(f[2], -x1, cscale(f[0], x3));
   cf[2] = cfma(f[0], -x2, cscale(f[1], x1));
+  cpx<R> u[3], ph[3];
 #pragma unroll
   for (int l = 0; l < 3; ++l) {
-    const cpx<R> Pf = cfma(xf, -(xi[l] * ik2), f[l]);
-    const cpx<R> Pg = cfma(xg, -(xi[l] * ik2), g[l]);
-    const cpx<R> tu = cfma(Pf, b, cmuli(cscale(cg[l], twok)));
-    const cpx<R> tp = cfma(Pg, a, cmuli(cscale(cf[l], twok)));
+    u[l] = cfma(f[l], u_f, cfma(xf, xi[l] * u_x, cmuli(cscale(cg[l], c_i))));
+    ph[l] = cfma(g[l], p_g, cfma(xg, xi[l] * p_x, cmuli(cscale(cf[l], c_i))));
+  }
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
     __align__(16) cpx<R> q[4];
-    q[0] = cfma(tu, iD, cscale(xf, xi[l] * iL_u));
-    q[1] = cmuli(cscale(q[0], x3));
-    q[2] = cfma(tp, iD, cscale(xg, xi[l] * iL_p));
-    q[3] = cmuli(cscale(q[2], x3));
+    q[0] = u[l];
+    q[1] = l == 0   ? cfma(cmuli(u[0]), x3, cmake<R>(-ph[1].x, -ph[1].y))
+           : l == 1 ? cfma(cmuli(u[1]), x3, ph[0])
+                    : cscale(cmuli(u[2]), x3);
+    q[2] = ph[l];
+    q[3] = cscale(cmuli(ph[l]), x3);
 #pragma unroll
     for (int i = 0; i < (int)sizeof(q) / 16; ++i)
       reinterpret_cast<Piece*>(v + 4 * l)[i] = reinterpret_cast<const Piece*>(q)[i];

@@ -60,6 +60,20 @@ constexpr size_t kSmemBudget = kSmemOptin - kSmemStaticReserve;
 // real for a real row and its imaginary part is ignored).  Tiles are AoS:
 // point k of line (rr, c) at [(rr M + k) 18 + c].
 
+// s + i conj(w) d, the packed pre-step of a pair a, b (s = a + b, d = a - b,
+// w = W_N1^k), and (s - i w d) / 2, the post-step.  The product enters the sum
+// by fused multiply-adds: one rounding less than forming it first.
+template <class R>
+__device__ __forceinline__ cpx<R> packed_pre(cpx<R> a, cpx<R> b, cpx<R> w) {
+  const cpx<R> s = cadd(a, b), d = csub(a, b);
+  return cmake<R>(fma(w.y, d.x, fma(-w.x, d.y, s.x)), fma(w.y, d.y, fma(w.x, d.x, s.y)));
+}
+template <class R>
+__device__ __forceinline__ cpx<R> packed_post(cpx<R> a, cpx<R> b, cpx<R> w) {
+  const cpx<R> s = cadd(a, b), d = csub(a, b);
+  return cmake<R>(R(0.5) * fma(w.y, d.x, fma(w.x, d.y, s.x)), R(0.5) * fma(w.y, d.y, fma(-w.x, d.x, s.y)));
+}
+
 __device__ __forceinline__ int div_m(int q, int M, int msh) { return msh >= 0 ? (q >> msh) : (q / M); }
 
 template <class R>
@@ -74,9 +88,7 @@ __device__ __forceinline__ void x_inverse_pre(const cpx<R>* X, cpx<R>* Z, int ro
     cpx<R> a = x[k * 18];
     if (k == 0) a.y = R(0);
     const cpx<R> b = (k == 0) ? cmake<R>(R(0), R(0)) : cconj(x[(M - k) * 18]);
-    cpx<R> w = tw[k];
-    w.y = -w.y;  // W_N^-k
-    Z[idx] = cadd(cadd(a, b), cmuli(cmul(w, csub(a, b))));
+    Z[idx] = packed_pre(a, b, tw[k]);
   }
 }
 
@@ -102,9 +114,7 @@ __device__ __forceinline__ void stage_first_inv_packed(const cpx<R>* __restrict_
       cpx<R> a = x[k * 18];
       if (k == 0) a.y = R(0);
       const cpx<R> b = (k == 0) ? cmake<R>(R(0), R(0)) : cconj(x[(M - k) * 18]);
-      cpx<R> w = tw[k];
-      w.y = -w.y;  // W_N^-k
-      v[r] = cadd(cadd(a, b), cmuli(cmul(w, csub(a, b))));
+      v[r] = packed_pre(a, b, tw[k]);
     }
     if constexpr (RADIX == 3) dft3<R, +1>(v);
     else if constexpr (RADIX == 4) dft4<R, +1>(v);
@@ -144,9 +154,7 @@ __device__ __forceinline__ void x_inv_first(const cpx<R>* X, cpx<R>* out, int ro
         a.y = R(0);
         b = cmake<R>(R(0), R(0));
       }
-      cpx<R> w = tw[k];
-      w.y = -w.y;  // W_N^-k
-      v[r] = cadd(cadd(a, b), cmuli(cmul(w, csub(a, b))));
+      v[r] = packed_pre(a, b, tw[k]);
     }
     dft<R, +1, RADIX>(v);
     cpx<R>* dst = out + (rr * M + j * RADIX) * 18 + c;
@@ -203,10 +211,7 @@ __device__ __forceinline__ void x_fwd_last(const cpx<R>* in, cpx<R>* X, int rows
       dft<R, -1, RADIX>(v);
     };
     auto post = [&](int k, cpx<R> a, cpx<R> zp) {
-      const cpx<R> b = cconj(zp);
-      const cpx<R> sm = cadd(a, b), df = csub(a, b);
-      const cpx<R> wd = cmul(tw[k], df);
-      dst[k * 18] = cmake<R>(R(0.5) * (sm.x + wd.y), R(0.5) * (sm.y - wd.x));
+      dst[k * 18] = packed_post(a, cconj(zp), tw[k]);
     };
     cpx<R> v[RADIX];
     butterfly(u, v);
@@ -347,10 +352,7 @@ __device__ __forceinline__ void x_forward_post(const cpx<R>* Z, cpx<R>* X, int r
     const cpx<R>* z = Z + rr * M * 18 + c;
     cpx<R> a = z[k * 18];
     cpx<R> b = cconj(z[(k == 0 ? 0 : M - k) * 18]);
-    cpx<R> s = cadd(a, b), d = csub(a, b);
-    cpx<R> wd = cmul(tw[k], d);
-    // (s - i wd) / 2
-    X[idx] = cmake<R>(R(0.5) * (s.x + wd.y), R(0.5) * (s.y - wd.x));
+    X[idx] = packed_post(a, b, tw[k]);
   }
 }
 
@@ -382,10 +384,7 @@ __device__ __forceinline__ void x_forward_last_post(const cpx<R>* __restrict__ i
     };
     // X[k] = (s - i W_N1^k d) / 2, s = Z[k] + conj(Z[M - k]), d = Z[k] - conj(Z[M - k])
     auto post = [&](int k, cpx<R> a, cpx<R> zp) {
-      const cpx<R> b = cconj(zp);
-      const cpx<R> sm = cadd(a, b), df = csub(a, b);
-      const cpx<R> wd = cmul(tw[k], df);
-      dst[k * LN] = cmake<R>(R(0.5) * (sm.x + wd.y), R(0.5) * (sm.y - wd.x));
+      dst[k * LN] = packed_post(a, cconj(zp), tw[k]);
     };
     cpx<R> v[RADIX];
     butterfly(u, v);

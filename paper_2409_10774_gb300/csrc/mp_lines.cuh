@@ -9,11 +9,15 @@
 //   A_l = i (x1 tau_1l + x2 tau_2l),                 T_l = tau_3l,
 //   B_l = i (x1 mu_1l + x2 mu_2l) + (eps : tau)_l,   M_l = mu_3l,
 // and the z pass, after its forward transform, forms f_l = A_l + i x3 T_l and
-// g_l = B_l + i x3 M_l.  It hands back u_l, i x3 u_l, phi_l, i x3 phi_l, from
+// g_l = B_l + i x3 M_l.  It hands back u_l, e_3l, phi_l, gamma_l3, from
 // which the inverse y pass forms the 18 components of (e~, gamma~) while it
 // reads them.  The z pass so transforms, reads and writes 12 values per point
 // instead of 18, and the passes move 84 complex values per point instead of
-// 108.  The 12 values sit in the first slots of the point's 18, l-major (the four
+// 108.  A_l, B_l are rounded before the z transform and i x1 u_l, i x2 u_l
+// meet phi_m only after it; fused multiply-adds here, in the operator and in
+// the packed x steps make up for that: on random FP32 fields the strain of a
+// 64^3 cell is 2.49e-7 off its 64-bit value (2.61e-7 without them, 2.50e-7
+// with all 18 fields through z).  The 12 values sit in the first slots of the point's 18, l-major (the four
 // values of one l are 16-byte pieces).  Cells with N2 = 1 have no y
 // pass; their z pass takes all 18.
 //
@@ -239,7 +243,7 @@ __device__ __forceinline__ void y_forward_tile(const CellDev<R>& c, long long ti
       cpx<R> o[4];
       o[0] = cmake<R>(-(ta.y * x1 + tb.y * x2), ta.x * x1 + tb.x * x2);
       o[1] = v[6 + l];
-      o[2] = cmake<R>(rot.x - (ma.y * x1 + mb.y * x2), rot.y + (ma.x * x1 + mb.x * x2));
+      o[2] = cmake<R>(fma(-mb.y, x2, fma(-ma.y, x1, rot.x)), fma(mb.x, x2, fma(ma.x, x1, rot.y)));
       o[3] = v[15 + l];
       store4(dst, o);
       v += dp * 18;
@@ -252,11 +256,11 @@ __device__ __forceinline__ void y_forward_tile(const CellDev<R>& c, long long ti
 
 // One line's reader of the 12 values after the z pass:
 //   e_kl = i xi_k u_l + eps_lkm phi_m,   gamma_kl = i xi_l phi_k,
-// where slot 4l + 1 holds i x3 u_l and slot 4k + 3 holds i x3 phi_k.  The
+// where slot 4l + 1 holds e_3l and slot 4k + 3 holds gamma_k3 as they are.  The
 // kinds are selected, not branched on (a warp holds lines of every kind).
 template <class R, int N>
 struct StrainReader {
-  const cpx<R>*w, *ph;  // u_l, phi_k or their x3 multiples; phi_m
+  const cpx<R>*w, *ph;  // u_l, phi_k or the value itself; phi_m
   const R* xi;          // x2 of the points
   R x1, sgn;            // sign of phi_m, 0 for none
   int der;              // axis of the derivative
@@ -264,7 +268,8 @@ struct StrainReader {
     constexpr int step = first_step<N>();
     const cpx<R> a = w[r * step * 12], b = ph[r * step * 12];
     const R f = der == 0 ? x1 : xi[r * step];
-    return cmake<R>(fma(sgn, b.x, der == 2 ? a.x : -(a.y * f)), fma(sgn, b.y, der == 2 ? a.y : a.x * f));
+    const cpx<R> d = cmake<R>(fma(-a.y, f, sgn * b.x), fma(a.x, f, sgn * b.y));
+    return der == 2 ? a : d;
   }
 };
 
@@ -289,7 +294,7 @@ __device__ __forceinline__ void y_inverse_tile(const CellDev<R>& c, long long ti
         StrainReader<R, N> s;
         s.der = is_e ? k : l;
         s.w = v + (is_e ? 4 * l : 4 * k + 2) + (s.der == 2 ? 1 : 0);
-        const bool rot = is_e && k != l;
+        const bool rot = is_e && k != l && k != 2;
         s.ph = rot ? v + 4 * (3 - k - l) + 2 : s.w;
         s.sgn = !rot ? R(0) : (l == (k + 1) % 3) ? R(-1) : R(1);
         s.x1 = c.n1 == 1 ? R(0) : c.two_pi_over_L[0] * (R)kx;
