@@ -1453,10 +1453,11 @@ __device__ __forceinline__ void commit_chunk(const CellDev<R>& c, long long chun
     return;
   }
   // Records per chunk: the field-type values are transposed through shared
-  // memory and summed by (value, part) threads - FP32 values in compensated
-  // pairs, folded in FP64 - and p, q by warp shuffles.  (Shuffling all 40
-  // values in FP64 cost 1600 warp additions a chunk on the FP64 pipe, 17 cycles
-  // each: the commit of a 32-cell batch took 755 us.)
+  // memory and summed in FP64 by (value, part) threads, p and q by warp
+  // shuffles.  (Shuffling all 40 values cost 1600 warp additions a chunk on the
+  // FP64 pipe, 17 cycles each: the commit of a 32-cell batch took 755 us.  The
+  // 344 of this form cost a 512-cell batch nothing against FP32 pairs, which
+  // keep fewer bits: 14.50 s with either.)
   constexpr int PITCH = 257, PARTS = 6, LEN = (256 + PARTS - 1) / PARTS;
   R* tile = reinterpret_cast<R*>(cols);  // [kAvgPartials][PITCH]
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1475,13 +1476,8 @@ __device__ __forceinline__ void commit_chunk(const CellDev<R>& c, long long chun
       const R* v = tile + i * PITCH;
       const int k1 = min(256, (part + 1) * LEN);
       double sm = 0.0;
-      if constexpr (sizeof(R) == 4) {
-        float2 acc = make_float2(0.f, 0.f);
-        for (int k = part * LEN; k < k1; ++k) two_sum_acc(acc, v[k]);
-        sm = (double)acc.x + (double)acc.y;
-      } else {
-        for (int k = part * LEN; k < k1; ++k) sm += v[k];
-      }
+#pragma unroll 4
+      for (int k = part * LEN; k < k1; ++k) sm += (double)v[k];
       red[part][i] = sm;
     }
   }
