@@ -366,7 +366,8 @@ def run_ours(args, rank, world, local_rank):
                    "gbs": (abytes[k] / (prof[k][0] / prof[k][1] / 1e3) / 1e9)
                    if (k in abytes and prof[k][1] and prof[k][0] > 0) else None}
                for k in KERNEL_CLASSES}
-    launches = int(sum(v[1] for v in prof.values()))
+    # (the reductions run inside pass A's launches)
+    launches = int(sum(v[1] for k, v in prof.items() if k != "reduce"))
 
     # ---------------- plain FP64 GPU solver on the same workload (speed-up base)
     fp64 = None

@@ -235,7 +235,8 @@ mp_status mp_rve_config(const mp_rve* rve, int32_t* cfg, int32_t n);
 #define MP_KC_GREEN_Z 1   /* z forward + Green operator + z inverse pass                */
 #define MP_KC_FFT_Y_INV 2 /* y-direction inverse transform pass                         */
 #define MP_KC_PASS_A 3    /* x inverse, Algorithm 1, error partials, polarization, x fwd */
-#define MP_KC_REDUCE 4    /* iteration error reduction (part of pass A: no launches)      */
+#define MP_KC_REDUCE 4    /* iteration error reduction, by pass A's last blocks: counted  */
+                          /* once an iteration, its time not in MP_KC_PASS_A's           */
 #define MP_KC_START 5     /* increment start: initial state, predictor pass              */
 #define MP_KC_COMMIT 6    /* commit of a converged increment and homogenized averages    */
 #define MP_KC_SPECTRAL 7  /* fused pass: y fwd, z fwd, Green operator, z inv, y inv       */
@@ -244,8 +245,9 @@ mp_status mp_rve_config(const mp_rve* rve, int32_t* cfg, int32_t n);
 /* Cells whose y and z lengths are 256 (FP32 fields) run classes 0-2 as the
  * one fused launch of class 7; other cells run classes 0-2.
  * Enable / disable per-kernel CUDA-event timing of mp_rve_run (events
- * recorded on the run's stream around every launch of every class; the
- * host waits for each increment's commit while enabled).  Launch counts are
+ * recorded on the run's stream around every launch of every class, device
+ * time stamps around the reduction; the host waits for each increment's
+ * commit while enabled).  Launch counts are
  * kept for every class regardless. */
 mp_status mp_rve_profile(mp_rve* rve, int32_t enable);
 /* Accumulated milliseconds (every class, while enabled) and launch counts

@@ -31,6 +31,12 @@ __device__ __forceinline__ R signed_freq_scale(int k, int n, R two_pi_over_L) {
   return two_pi_over_L * (R)s;
 }
 
+__device__ __forceinline__ unsigned long long globaltimer_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 // col / kx of a column index (< 2^18, kx <= 2^8): exact by the multiplier
 // ceil(2^32 / kx), whose excess kx_magic kx - 2^32 < kx keeps col times it
 // below 2^32.

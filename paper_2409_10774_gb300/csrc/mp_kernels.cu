@@ -1089,6 +1089,8 @@ __device__ __forceinline__ void fold_records(const double* __restrict__ records,
 // (stag > 0) the stagnation watch (stall_step with window stag) has not
 // tripped: out[7], out[8] hold the last low and its iteration, out[10] the
 // longest gap between lows, out[9] = 1 records a stop by the watch.
+// out[11]: nanoseconds from the end of the last block's items to here, the
+// reduction's share of pass A.
 constexpr int kTailGroup = 16;
 template <class R>
 __device__ void finish_blocks(const CellDev<R>& c, double* partials, const double* acc, const ErrTail& tail) {
@@ -1096,6 +1098,7 @@ __device__ void finish_blocks(const CellDev<R>& c, double* partials, const doubl
   __shared__ double part[SPLIT][NQ], s[NQ];
   __shared__ FinishScratch fin;
   __shared__ int last;
+  const unsigned long long entered = globaltimer_ns();
   const int t = threadIdx.x, grid = (int)gridDim.x, group = (int)blockIdx.x / kTailGroup;
   const int groups = (grid + kTailGroup - 1) / kTailGroup;
   double* records = partials + (long long)kTailRecords * NQ;  // the blocks', after the groups'
@@ -1135,6 +1138,7 @@ __device__ void finish_blocks(const CellDev<R>& c, double* partials, const doubl
   if (!arrive(tail.counters + kTailRecords, groups)) return;
   fold(partials, groups);
   if (t < 32) finish_err<R>(c, s, tail.err_kind, tail.out, fin);
+  if (t == 0) tail.out[11] = (double)(globaltimer_ns() - entered);
   if (t == 0 && tail.loop) {
     double* out = tail.out;
     const int it = (int)out[6] + 1;
