@@ -24,6 +24,7 @@
 #include "mp_device.cuh"
 #include "mp_fft.cuh"
 #include "mp_lines.cuh"
+#include "mp_plan.cuh"
 #include "mp_tma.cuh"
 
 namespace mp {
@@ -1989,35 +1990,9 @@ LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted, bool sh
   L.grid_a = std::min(grid_for<R>((const void*)k_pass_a<R, kIter, false>, L.threads_a, smem_a, items, nsm),
                       kPassABlocks * nsm);
   L.grid_max = kPassABlocks * nsm;
-  // Columns per y / z tile: about 256 (FP32) or 128 (FP64) points for cells
-  // launched together.  A cell alone takes, in FP64, fewer where that would
-  // not give every SM two tiles (16^3: the three passes took 106 us in 8 tiles
-  // of 16 columns, 40 us in 128 of one; fewer columns than that only leave
-  // lanes of the FP64 pipe idle), and in FP32 the size that ends soonest: the
-  // tiles run in waves of what the SMs hold, and a wave costs its tile's
-  // points plus a fixed latency, about 100 points' worth (64^3: 11.9 us a pass
-  // in 512 tiles of four columns, which is one wave and an eighth, 10.6 us in
-  // 2048 of one).
-  auto columns = [&](int n, long long ncols) {
-    const int full = std::max(1, (sizeof(R) == 4 ? 256 : 128) / n);
-    if (shared) return full;
-    if (sizeof(R) == 8) return (int)std::min<long long>(full, std::max<long long>(1, ncols / (2 * nsm)));
-    int best = full;
-    double best_cost = INFINITY;
-    for (int cols = full; cols >= 1; --cols) {
-      const long long tiles = (ncols + cols - 1) / cols;
-      const long long slots = (long long)nsm * std::max(1, 800 / (cols * n));
-      const double cost = (double)((tiles + slots - 1) / slots) * (cols * n + 100.0);
-      if (cost < 0.97 * best_cost) {
-        best = cols;
-        best_cost = cost;
-      }
-    }
-    return best;
-  };
   CellDev<R> t = c;
-  t.cols_y = L.cols_y = columns(c.n2, (long long)c.n3 * c.kx);
-  t.cols_z = L.cols_z = columns(c.n3, (long long)c.n2 * c.kx);
+  t.cols_y = L.cols_y = tile_columns(c.n2, (long long)c.n3 * c.kx, sizeof(R) == 8, shared, nsm);
+  t.cols_z = L.cols_z = tile_columns(c.n3, (long long)c.n2 * c.kx, sizeof(R) == 8, shared, nsm);
   if (!shared) {
     if (c.n2 > 1) L.grid_y = std::min(line_grid<R, kYForward>(t, nsm), line_grid<R, kYInverse>(t, nsm));
     L.grid_z = c.n2 == 1 ? line_grid<R, kZFull>(t, nsm) : line_grid<R, kZReduced>(t, nsm);

@@ -13,6 +13,40 @@
 
 namespace mp {
 
+// Columns of length n per y / z tile, of `ncols` in all, on `nsm` SMs.  Cells
+// launched together (shared) take about 256 points (FP32) or 128 (FP64).  A
+// cell alone takes, in FP64, fewer where that would not give every SM two
+// tiles (16^3: the three passes took 106 us in 8 tiles of 16 columns, 40 us in
+// 128 of one; fewer columns than that only leave lanes of the FP64 pipe idle),
+// and in FP32 the size that ends soonest: the tiles run in waves of what the
+// SMs hold - about 800 points each, in at most 32 blocks - and a wave costs its
+// tile's points plus a fixed latency, about 100 points' worth (64^3: 11.9 us a
+// pass in 512 tiles of four columns, which is one wave and an eighth, 10.6 us
+// in 2048 of one; 256 x 128 x 8: the z pass 26 us in tiles of one column, 17 us
+// in tiles of two, which an unlimited number of blocks would not be given).
+constexpr int kTileBlocks = 32;  // blocks an SM holds at most
+inline int tile_columns(int n, long long ncols, bool fp64, bool shared, int nsm) {
+  const int full = n < (fp64 ? 128 : 256) ? (fp64 ? 128 : 256) / n : 1;
+  if (shared) return full;
+  if (fp64) {
+    const long long most = ncols / (2 * nsm) > 1 ? ncols / (2 * nsm) : 1;
+    return full < most ? full : (int)most;
+  }
+  int best = full;
+  double best_cost = INFINITY;
+  for (int cols = full; cols >= 1; --cols) {
+    int blocks = 800 / (cols * n);
+    blocks = blocks < 1 ? 1 : blocks > kTileBlocks ? kTileBlocks : blocks;
+    const long long tiles = (ncols + cols - 1) / cols, slots = (long long)nsm * blocks;
+    const double cost = (double)((tiles + slots - 1) / slots) * (cols * n + 100.0);
+    if (cost < 0.97 * best_cost) {
+      best = cols;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 // Radix sequence of the packed x axis' complex transform of length m = 2^a 3^b
 // (for the lengths without compile-time stages): powers of two in as few
 // radix-8 stages as possible, radix-3 stages last.
