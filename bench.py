@@ -62,7 +62,7 @@ def algorithmic_bytes(n, precision=1):
 # Host-only sources (entry points, the batched engine's host loop, the static
 # entry point, host helpers): a change there leaves the kernels' DRAM traffic
 # as it was, so they do not enter the hash that dates a traffic capture.
-HOST_ONLY_SOURCES = ("mp_api.cu", "mp_batch.cu", "mp_static.cu", "mp_host.cuh")
+HOST_ONLY_SOURCES = ("mp_api.cu", "mp_batch.cu", "mp_static.cu", "mp_host.cuh", "mp_limits.cuh")
 
 
 def _source_hash():

@@ -15,14 +15,11 @@
 
 #include <algorithm>
 #include <cmath>
-#include <map>
-#include <mutex>
-#include <set>
-#include <tuple>
 
 #include "mp_constitutive.cuh"
 #include "mp_device.cuh"
 #include "mp_fft.cuh"
+#include "mp_limits.cuh"
 #include "mp_lines.cuh"
 #include "mp_plan.cuh"
 #include "mp_tma.cuh"
@@ -1723,64 +1720,35 @@ template <class R>
 constexpr size_t kCommitTile = (size_t)kAvgPartials * 257 * sizeof(R);  // multi-cell commit, a chunk's values
 constexpr size_t kCommitSmem = (size_t)kAvgPartials * 256 * sizeof(double);  // single-cell commit columns
 
-// Raise the dynamic shared-memory limit of the kernels launched without a
-// resident_blocks call to what their static shared memory leaves of the
-// opt-in maximum (at least kSmemBudget).
-template <class R>
-static cudaError_t set_smem_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
-  // tiles: kernels whose tiles may take up to kSmemBudget (their static shared
-  // memory must fit the reserve)
-  auto raise = [&](const void* fn, bool tiles = true) {
-    if (e != cudaSuccess) return;
+namespace {
+struct RuntimeApi {
+  using Error = cudaError_t;
+  static constexpr Error ok = cudaSuccess, invalid = cudaErrorInvalidValue;
+  static Error device(int& dev) { return cudaGetDevice(&dev); }
+  static Error static_smem(const void* fn, size_t& bytes) {
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, fn);
-    if (e != cudaSuccess) return;
-    if (tiles && fa.sharedSizeBytes > kSmemStaticReserve) {
-      e = cudaErrorInvalidValue;
-      return;
-    }
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kSmemOptin - fa.sharedSizeBytes));
-  };
-  raise((const void*)k_pass_a<R, kIter, false>);
-  raise((const void*)k_pass_a<R, kStart, false>);
-  raise((const void*)k_pass_a<R, kXFwd, false>);
-  raise((const void*)k_pass_a<R, kXInv, false>);
-  raise((const void*)k_pass_a<R, kIter, true>);
-  raise((const void*)k_pass_a<R, kStart, true>);
-  raise((const void*)k_commit<R, false>, false);
-  raise((const void*)k_commit<R, true>, false);
-  if (e == cudaSuccess) done = true;
-  return e;
+    const Error e = cudaFuncGetAttributes(&fa, fn);
+    bytes = e == cudaSuccess ? fa.sharedSizeBytes : 0;
+    return e;
+  }
+  static Error raise(const void* fn, size_t bytes) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  }
+  static Error occupancy(const void* fn, int threads, size_t smem, int& blocks) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, threads, smem);
+  }
+};
+
+KernelLimits<RuntimeApi>& kernel_limits() {
+  static KernelLimits<RuntimeApi> limits(kSmemOptin, kSmemStaticReserve);
+  return limits;
 }
+}  // namespace
+
+cudaError_t raise_smem(const void* fn, bool tiled) { return kernel_limits().raise(fn, tiled); }
 
 int resident_blocks(const void* fn, int threads, size_t smem) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, const void*, int, size_t>, int> known;
-  static std::set<std::pair<int, const void*>> raised;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  std::lock_guard<std::mutex> lock(mu);
-  const auto key = std::make_tuple(dev, fn, threads, smem);
-  const auto it = known.find(key);
-  if (it != known.end()) return it->second;
-  if (!raised.count({dev, fn})) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kSmemOptin - fa.sharedSizeBytes)) != cudaSuccess)
-      return 1;
-    raised.insert({dev, fn});
-  }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess) return 1;
-  if (per_sm < 1) per_sm = 1;
-  if (known.size() >= 4096) known.clear();
-  known[key] = per_sm;
-  return per_sm;
+  return std::max(1, kernel_limits().resident(fn, false, threads, smem));
 }
 
 template <class R>
@@ -1803,7 +1771,7 @@ cudaError_t launch_green_z(const LaunchCfg& L, const CellDev<R>& c, cudaStream_t
 template <class R>
 cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* partials, const ErrTail& tail,
                                cudaStream_t st) {
-  cudaError_t e = set_smem_attrs<R>();
+  const cudaError_t e = raise_smem((const void*)k_pass_a<R, kIter, false>, true);
   if (e != cudaSuccess) return e;
   ErrTail t = tail;
   t.counters = reinterpret_cast<unsigned*>(partials + (size_t)(kTailRecords + L.grid_max) * kErrPartials);
@@ -1814,7 +1782,7 @@ cudaError_t launch_pass_a_iter(const LaunchCfg& L, const CellDev<R>& c, double* 
 
 template <class R>
 cudaError_t launch_start(const LaunchCfg& L, const CellDev<R>& c, int first, cudaStream_t st) {
-  cudaError_t e = set_smem_attrs<R>();
+  const cudaError_t e = raise_smem((const void*)k_pass_a<R, kStart, false>, true);
   if (e != cudaSuccess) return e;
   if (first) k_init<R, false><<<L.grid_v, 256, 0, st>>>(c, Work<R>{});
   k_pass_a<R, kStart, false><<<L.grid_a, L.threads_a, smem_pass_a<R>(c.n1, c.rows_a), st>>>(
@@ -1825,6 +1793,8 @@ cudaError_t launch_start(const LaunchCfg& L, const CellDev<R>& c, int first, cud
 template <class R>
 cudaError_t launch_commit(const LaunchCfg& L, const CellDev<R>& c, double* partials, double* avg_out,
                           cudaStream_t st) {
+  const cudaError_t e = raise_smem((const void*)k_commit<R, false>, false);
+  if (e != cudaSuccess) return e;
   k_commit<R, false><<<L.grid_v, 256, kCommitSmem, st>>>(c, Work<R>{}, partials);
   k_reduce_avg<<<1, kFoldThreads, 0, st>>>(partials, L.grid_v, c.inv_nvox, avg_out, c.tmean);
   return cudaGetLastError();
@@ -1833,7 +1803,7 @@ cudaError_t launch_commit(const LaunchCfg& L, const CellDev<R>& c, double* parti
 // ------------------------------------------------------------------ multi-cell launches
 template <class R>
 cudaError_t launch_multi_iteration(const MultiCfg<R>& m, cudaStream_t st) {
-  cudaError_t e = set_smem_attrs<R>();
+  cudaError_t e = raise_smem((const void*)k_pass_a<R, kIter, true>, true);
   if (e != cudaSuccess) return e;
   if (m.items_y > 0 && (e = launch_line_multi<R, kYForward>(m.wy, m.grid_y, m.smem_y, st)) != cudaSuccess) return e;
   if (m.items_z > 0 && (e = launch_line_multi<R, kZReduced>(m.wz, m.grid_z, m.smem_z, st)) != cudaSuccess) return e;
@@ -1847,7 +1817,7 @@ cudaError_t launch_multi_iteration(const MultiCfg<R>& m, cudaStream_t st) {
 
 template <class R>
 cudaError_t launch_multi_start(const MultiCfg<R>& m, cudaStream_t st) {
-  cudaError_t e = set_smem_attrs<R>();
+  const cudaError_t e = raise_smem((const void*)k_pass_a<R, kStart, true>, true);
   if (e != cudaSuccess) return e;
   if (m.items_v0 > 0) k_init<R, true><<<m.grid_v0, 256, 0, st>>>(CellDev<R>{}, m.wv0);
   if (m.items_s > 0)
@@ -1858,7 +1828,7 @@ cudaError_t launch_multi_start(const MultiCfg<R>& m, cudaStream_t st) {
 
 template <class R>
 cudaError_t launch_multi_commit(const MultiCfg<R>& m, cudaStream_t st) {
-  const cudaError_t e = set_smem_attrs<R>();
+  const cudaError_t e = raise_smem((const void*)k_commit<R, true>, false);
   if (e != cudaSuccess) return e;
   if (m.items_v > 0) k_commit<R, true><<<m.grid_v, 256, kCommitTile<R>, st>>>(CellDev<R>{}, m.wv, nullptr);
   if (m.wv.n_act > 0) k_reduce_avg_multi<R><<<m.wv.n_act, kFoldThreads, 0, st>>>(m.wv);
@@ -1867,7 +1837,6 @@ cudaError_t launch_multi_commit(const MultiCfg<R>& m, cudaStream_t st) {
 
 template <class R>
 void multi_grids(MultiCfg<R>& m, int nsm) {
-  set_smem_attrs<R>();
   m.grid_y = std::min(line_multi_grid<R, kYForward>(m.items_y, m.smem_y, nsm),
                       line_multi_grid<R, kYInverse>(m.items_y, m.smem_y, nsm));
   m.grid_z = line_multi_grid<R, kZReduced>(m.items_z, m.smem_z, nsm);
@@ -1891,7 +1860,8 @@ cudaError_t launch_fields(const LaunchCfg& L, const CellDev<R>& c, int from_elas
 template <class R>
 cudaError_t launch_green_apply(const LaunchCfg& L, const CellDev<R>& c, const R* tau, const R* mu,
                                R* e_out, R* g_out, cudaStream_t st, int* ctl, int nsm) {
-  cudaError_t e = set_smem_attrs<R>();
+  cudaError_t e = raise_smem((const void*)k_pass_a<R, kXFwd, false>, true);
+  if (e == cudaSuccess) e = raise_smem((const void*)k_pass_a<R, kXInv, false>, true);
   if (e != cudaSuccess) return e;
   const size_t sa = smem_pass_a<R>(c.n1, c.rows_a);
   k_pass_a<R, kXFwd, false><<<L.grid_a, L.threads_a, sa, st>>>(c, Work<R>{}, nullptr, tau, mu, nullptr, nullptr, ErrTail{});
@@ -1961,7 +1931,6 @@ template cudaError_t launch_convert<double, float>(const double*, float*, long l
 
 template <class R>
 LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted, bool shared) {
-  set_smem_attrs<R>();
   LaunchCfg L;
   // rows per pass-A item: about 256 voxels per block (FP64: 128, see below) or
   // as asked, within the shared-memory budget; a cell alone takes fewer rows

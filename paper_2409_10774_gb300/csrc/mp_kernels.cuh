@@ -38,10 +38,10 @@ void use_launch_cfg(CellDev<R>& c, const LaunchCfg& L) {
 template <class R>
 bool sizes_fit(int n1, int n2, int n3);
 
-// Blocks of `fn` an SM of the current device holds (at least 1), after letting
-// it use the shared memory its static part leaves of the opt-in maximum.
-// Answers are kept per kernel and shape: asking the runtime costs microseconds
-// and the component calls ask each time.
+// Lets `fn` use the shared memory its static part leaves of the opt-in maximum
+// on the current device (KernelLimits; tiled: the static part must fit the
+// reserve), and the blocks of it an SM holds, at least 1, with the limit raised.
+cudaError_t raise_smem(const void* fn, bool tiled);
 int resident_blocks(const void* fn, int threads, size_t smem);
 
 // The line passes (mp_lines.cuh): y forward, y inverse, and z with the Green
