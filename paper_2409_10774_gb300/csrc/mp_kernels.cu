@@ -1747,13 +1747,13 @@ KernelLimits<RuntimeApi>& kernel_limits() {
 
 cudaError_t raise_smem(const void* fn, bool tiled) { return kernel_limits().raise(fn, tiled); }
 
-int resident_blocks(const void* fn, int threads, size_t smem) {
-  return std::max(1, kernel_limits().resident(fn, false, threads, smem));
+int resident_blocks(const void* fn, int threads, size_t smem, bool tiled) {
+  return std::max(1, kernel_limits().resident(fn, tiled, threads, smem));
 }
 
 template <class R>
-int grid_for(const void* fn, int threads, size_t smem, long long work, int nsm) {
-  const long long g = std::min<long long>(work, (long long)resident_blocks(fn, threads, smem) * nsm);
+int grid_for(const void* fn, int threads, size_t smem, long long work, int nsm, bool tiled = true) {
+  const long long g = std::min<long long>(work, (long long)resident_blocks(fn, threads, smem, tiled) * nsm);
   return (int)std::max<long long>(g, 1);
 }
 
@@ -1904,7 +1904,7 @@ cudaError_t launch_radial_return(int nsm, long long count, const uint16_t* phase
   while (threads > 32 && count < (long long)threads * 2 * nsm) threads /= 2;
   const size_t smem = 54 * (size_t)threads * sizeof(R) + (dev_phases ? 0 : n_phases * sizeof(PhaseDev<R>));
   const void* fn = vec ? (const void*)k_radial_return_points<R, true> : (const void*)k_radial_return_points<R, false>;
-  const int grid = grid_for<R>(fn, threads, smem, (count + threads - 1) / threads, nsm);
+  const int grid = grid_for<R>(fn, threads, smem, (count + threads - 1) / threads, nsm, false);
   void* args[] = {&table, (void*)&dev_phases, &n_phases, &count, &P};
   return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, st);
 }
@@ -1973,10 +1973,10 @@ LaunchCfg make_launch_cfg(const CellDev<R>& c, int nsm, int rows_wanted, bool sh
 
 template <class R>
 bool sizes_fit(int n1, int n2, int n3) {
-  // a y / z tile holds at least one whole column: two copies of its 18 lines
-  // and one more of a line's length for the tables
-  auto column = [](int n) { return 37 * (size_t)n * sizeof(cpx<R>) + 16 * sizeof(long long); };
-  return smem_pass_a<R>(n1, 1) <= kSmemBudget && column(n2) <= kSmemBudget && column(n3) <= kSmemBudget;
+  // a y / z tile holds at least one whole column of 18 lines (the longest in
+  // FP64, 384, takes the whole budget)
+  return smem_pass_a<R>(n1, 1) <= kSmemBudget && smem_line<R>(n2, 1, 18) <= kSmemBudget &&
+         smem_line<R>(n3, 1, 18) <= kSmemBudget;
 }
 
 #define MP_INSTANTIATE(R)                                                                            \

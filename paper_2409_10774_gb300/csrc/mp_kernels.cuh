@@ -42,7 +42,7 @@ bool sizes_fit(int n1, int n2, int n3);
 // on the current device (KernelLimits; tiled: the static part must fit the
 // reserve), and the blocks of it an SM holds, at least 1, with the limit raised.
 cudaError_t raise_smem(const void* fn, bool tiled);
-int resident_blocks(const void* fn, int threads, size_t smem);
+int resident_blocks(const void* fn, int threads, size_t smem, bool tiled);
 
 // The line passes (mp_lines.cuh): y forward, y inverse, and z with the Green
 // operator on the reduced 12 fields or, for cells without a y pass, on all 18.

@@ -468,7 +468,7 @@ int line_grid(const CellDev<R>& c, int nsm) {
   if (!fn) return 1;
   const int threads = line_block<R, PASS>(n, cols);
   const long long tiles = PASS < kZReduced ? tiles_y(c) : tiles_z(c);
-  const long long most = (long long)resident_blocks(fn, threads, smem_line<R>(n, cols, PASS == kZReduced ? 12 : 18)) * nsm;
+  const long long most = (long long)resident_blocks(fn, threads, smem_line<R>(n, cols, PASS == kZReduced ? 12 : 18), true) * nsm;
   return (int)(tiles < most ? tiles : most);
 }
 
@@ -485,7 +485,7 @@ cudaError_t launch_line(const CellDev<R>& c, int grid, cudaStream_t st) {
 template <class R, int PASS>
 int line_multi_grid(long long items, size_t smem, int nsm) {
   const long long most =
-      (long long)resident_blocks((const void*)k_line_multi<R, PASS>, line_threads<R>(PASS), smem) * nsm;
+      (long long)resident_blocks((const void*)k_line_multi<R, PASS>, line_threads<R>(PASS), smem, true) * nsm;
   return (int)(items < 1 ? 1 : items < most ? items : most);
 }
 

@@ -368,7 +368,7 @@ constexpr size_t kSpecSmem = ((size_t)kStages * kTile + kN) * sizeof(cpx<float>)
                              2 * kStages * sizeof(uint64_t) + kStages * sizeof(SlotInfo);
 
 cudaError_t launch_spectral(const CellDev<float>& c, int* ctl, int nsm, cudaStream_t st) {
-  const int per_sm = resident_blocks((const void*)k_spectral, kBlock, kSpecSmem);
+  const int per_sm = resident_blocks((const void*)k_spectral, kBlock, kSpecSmem, true);
   // the blocks wait on one another's items: all must be resident at once
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(per_sm * nsm));
