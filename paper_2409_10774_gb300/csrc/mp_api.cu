@@ -247,13 +247,14 @@ mp_status validate_problem(const mp_problem* p, std::vector<long long>* counts_o
 
 // ------------------------------------------------------------------ plans and tables
 template <class R>
-mp_status make_axis(mp_ctx* ctx, int n, bool packed, AxisPlan<R>& p, DevBuf& tw, cudaStream_t st,
-                    std::vector<cpx<R>>& host_tw) {
-  axis_tables<R>(n, packed, p, host_tw);
+mp_status make_table(mp_ctx* ctx, int n, const cpx<R>*& table, DevBuf& tw, cudaStream_t st,
+                     std::vector<cpx<R>>& host_tw) {
+  host_tw.resize(n);
+  twiddle_table<R>(n, host_tw.data());
   mp_status s = dalloc(ctx, tw, sizeof(cpx<R>) * n);
   if (s != MP_OK) return s;
   MP_CK(ctx, cudaMemcpyAsync(tw.ptr, host_tw.data(), sizeof(cpx<R>) * n, cudaMemcpyHostToDevice, st));
-  p.tw = reinterpret_cast<const cpx<R>*>(tw.ptr);
+  table = reinterpret_cast<const cpx<R>*>(tw.ptr);
   return MP_OK;
 }
 
@@ -379,9 +380,10 @@ mp_status rve_setup(mp_rve* r, const mp_problem* p, cudaStream_t st) {
   std::vector<PhaseDev<R>> ph(p->n_phases);
   for (int k = 0; k < p->n_phases; ++k) ph[k] = phase_dev<R>(p->phases[k], p->precision == 2);
   std::vector<cpx<R>> t1, t2, t3;
-  if ((s = make_axis<R>(ctx, c.n1, true, c.px, r->twx, st, t1)) != MP_OK) return s;
-  if ((s = make_axis<R>(ctx, c.n2, false, c.py, r->twy, st, t2)) != MP_OK) return s;
-  if ((s = make_axis<R>(ctx, c.n3, false, c.pz, r->twz, st, t3)) != MP_OK) return s;
+  c.px = radix_plan(c.n1);
+  if ((s = make_table<R>(ctx, c.n1, c.tw[0], r->twx, st, t1)) != MP_OK) return s;
+  if ((s = make_table<R>(ctx, c.n2, c.tw[1], r->twy, st, t2)) != MP_OK) return s;
+  if ((s = make_table<R>(ctx, c.n3, c.tw[2], r->twz, st, t3)) != MP_OK) return s;
   MP_CK(ctx, cudaMemcpyAsync(r->phase.ptr, p->phase, sizeof(uint16_t) * (size_t)c.nvox,
                              cudaMemcpyHostToDevice, st));
   MP_CK(ctx, cudaMemcpyAsync(r->phases.ptr, ph.data(), sizeof(PhaseDev<R>) * ph.size(),
@@ -451,9 +453,10 @@ mp_status twin_setup(mp_rve* r, cudaStream_t st) {
   std::vector<PhaseDev<double>> ph(r->phases_host.size());
   for (size_t k = 0; k < ph.size(); ++k) ph[k] = phase_dev<double>(r->phases_host[k], false);
   std::vector<cpx<double>> t1, t2, t3;
-  if ((s = make_axis<double>(ctx, c.n1, true, c.px, r->twx64, st, t1)) != MP_OK) return s;
-  if ((s = make_axis<double>(ctx, c.n2, false, c.py, r->twy64, st, t2)) != MP_OK) return s;
-  if ((s = make_axis<double>(ctx, c.n3, false, c.pz, r->twz64, st, t3)) != MP_OK) return s;
+  c.px = radix_plan(c.n1);
+  if ((s = make_table<double>(ctx, c.n1, c.tw[0], r->twx64, st, t1)) != MP_OK) return s;
+  if ((s = make_table<double>(ctx, c.n2, c.tw[1], r->twy64, st, t2)) != MP_OK) return s;
+  if ((s = make_table<double>(ctx, c.n3, c.tw[2], r->twz64, st, t3)) != MP_OK) return s;
   MP_CK(ctx, cudaMemcpyAsync(r->phases64.ptr, ph.data(), sizeof(PhaseDev<double>) * ph.size(),
                              cudaMemcpyHostToDevice, st));
   r->L64 = make_launch_cfg<double>(c, ctx->nsm);
@@ -1463,10 +1466,10 @@ mp_status green_apply_impl(mp_ctx* ctx, const int32_t n[3], double h, const doub
   // tables) and one upload per call
   bool fused = false;
   if constexpr (sizeof(R) == 4) fused = spectral_fused_ok(c);
-  AxisPlan<R>* const plans[3] = {&c.px, &c.py, &c.pz};
+  c.px = radix_plan(c.n1);
   static thread_local __align__(16) unsigned char image[kImageBytes];
   size_t table[3];
-  const size_t image_bytes = operator_image<R>(n, plans, 4 + (fused ? spectral_ctl_ints(c.kx) : 0), image, table);
+  const size_t image_bytes = operator_image<R>(n, 4 + (fused ? spectral_ctl_ints(c.kx) : 0), image, table);
   const size_t spec_bytes = (sizeof(cpx<R>) * 18 * (size_t)c.nspec + 255) / 256 * 256;
   DevBuf buf;
   mp_status st = dalloc(ctx, buf, spec_bytes + image_bytes);
@@ -1474,7 +1477,7 @@ mp_status green_apply_impl(mp_ctx* ctx, const int32_t n[3], double h, const doub
   unsigned char* meta = static_cast<unsigned char*>(buf.ptr) + spec_bytes;
   c.spec = reinterpret_cast<cpx<R>*>(buf.ptr);
   c.status = reinterpret_cast<int*>(meta);
-  for (int a = 0; a < 3; ++a) plans[a]->tw = reinterpret_cast<const cpx<R>*>(meta + table[a]);
+  for (int a = 0; a < 3; ++a) c.tw[a] = reinterpret_cast<const cpx<R>*>(meta + table[a]);
   LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm);
   use_launch_cfg(c, L);
   int flag = 0;

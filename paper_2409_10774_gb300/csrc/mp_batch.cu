@@ -561,12 +561,13 @@ class Engine {
     }
     std::vector<PhaseDev<R>> ph(q->phases.size());
     for (size_t k = 0; k < ph.size(); ++k) ph[k] = phase_dev<R>(q->phases[k], q->precision == 2);
-    AxisPlan<R>* plans[3] = {&c.px, &c.py, &c.pz};
+    c.px = radix_plan(c.n1);
     std::vector<cpx<R>> tw[3];
     cudaError_t e = cudaSuccess;
     for (int a = 0; a < 3; ++a) {
-      axis_tables<R>(q->n[a], a == 0, *plans[a], tw[a]);
-      plans[a]->tw = reinterpret_cast<const cpx<R>*>(b + A.tw[a]);
+      tw[a].resize(q->n[a]);
+      twiddle_table<R>(q->n[a], tw[a].data());
+      c.tw[a] = reinterpret_cast<const cpx<R>*>(b + A.tw[a]);
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(b + A.tw[a], tw[a].data(), sizeof(cpx<R>) * q->n[a], cudaMemcpyHostToDevice, st_);
     }

@@ -92,17 +92,12 @@ struct RefDev {
   R lam, mu, kap, alpha, beta, gamma;
 };
 
-// FFT plan of one axis: length N, radix sequence for the complex transform of
-// length M (M = N / 2 for the packed real x-axis, M = N otherwise) and the
-// device twiddle table W_T^k = exp(-2 pi i k / T), k < T, with T = N.
-template <class R>
-struct AxisPlan {
-  int n;          // axis length
-  int m;          // complex transform length
-  int tstride;    // twiddle table stride: W_m^k = table[k * tstride]
+// Radix sequence of the packed x axis' complex transform, of length m = N1 / 2,
+// where its stages are not compile-time ones.
+struct RadixPlan {
+  int m;
   int nstages;
   int radix[10];
-  const cpx<R>* tw;  // table of length n (n >= 1)
 };
 
 // Loop control of one cell over a window of batched rounds: Algorithm 2's
@@ -147,7 +142,8 @@ struct CellDev {
   const uint16_t* phase;  // [nvox]
   const PhaseDev<R>* phases;
   RefDev<R> ref;
-  AxisPlan<R> px, py, pz;
+  RadixPlan px;
+  const cpx<R>* tw[3];    // twiddle tables of the axes: W_N^k = exp(-2 pi i k / N), k < N
   R E[9], G[9];           // prescribed averages of the current step
   int* status;            // device status word: bit 0 = a bounded wait expired
   int cols_y, cols_z;     // columns per tile of the y / z passes

@@ -255,17 +255,17 @@ __host__ __device__ constexpr int line_table(int n) { return (n + (n + 1) / 2 + 
 // values: the stages are free of shared-memory bank conflicts and need no
 // transposition on load or store.
 //
-// One Stockham stage of radix R (2, 3, 4, 8 or 16) with Ns = product of the radices already
+// One Stockham stage of radix R (2, 3, 4 or 8) with Ns = product of the radices already
 // applied: butterfly j of a line reads points j + r M / R (r < R), multiplies
 // point r by W_M^(r (j mod Ns) M / (Ns R)), takes the R-point DFT and writes
 // output r to point (j / Ns) Ns R + (j mod Ns) + r Ns.  The last stage leaves
 // natural order (no bit reversal).  The host orders radix-3 stages last, so
 // only those divide by a non-power-of-two Ns.
-// MAXR bounds the radices a kernel instantiates (8 keeps the 16-point
-// butterfly's registers out of kernels that never use it).
-template <class R, int DIR, int MAXR>
+// The packed x axis' table holds the 2 M roots: W_M^k = tw[2 k].
+template <class R, int DIR>
 __device__ void stage_aos(const cpx<R>* __restrict__ in, cpx<R>* __restrict__ out, int rows, int M,
-                          int radix, int Ns, const cpx<R>* __restrict__ tw, int tstride) {
+                          int radix, int Ns, const cpx<R>* __restrict__ tw) {
+  constexpr int MAXR = 8;
   const int nb = M / radix;
   const int total = rows * nb * 18;
   const int tstep = M / (Ns * radix);
@@ -292,17 +292,14 @@ __device__ void stage_aos(const cpx<R>* __restrict__ in, cpx<R>* __restrict__ ou
       if (r < radix) {
         cpx<R> x = src[(j + r * nb) * 18];
         const int e = r * kk * tstep;  // < M
-        v[r] = e == 0 ? x : cmul(x, twiddle<R, DIR>(tw, e * tstride));
+        v[r] = e == 0 ? x : cmul(x, twiddle<R, DIR>(tw, e * 2));
       }
     }
     switch (radix) {
       case 2: dft2<R, DIR>(v); break;
       case 3: dft3<R, DIR>(v); break;
       case 4: dft4<R, DIR>(v); break;
-      case 8: dft8<R, DIR>(v); break;
-      default:
-        if constexpr (MAXR >= 16) dft16<R, DIR>(v);
-        break;
+      default: dft8<R, DIR>(v); break;
     }
     cpx<R>* dst = out + rr * rs + c + (jq * Ns * radix + kk) * 18;
 #pragma unroll
@@ -312,53 +309,45 @@ __device__ void stage_aos(const cpx<R>* __restrict__ in, cpx<R>* __restrict__ ou
   }
 }
 
-// The same stage with the radix, Ns, the line length M and the twiddle stride
-// known at compile time (index arithmetic folds to shifts and constants, and
-// only the one butterfly is instantiated).  LN lines are interleaved point by
-// point (18 components of one column, or of several columns side by side).
-template <class R, int DIR, int RADIX, int NS, int M, int TSTRIDE, int LN = 18>
+// The same stage with the radix, Ns and the line length M known at compile time
+// (index arithmetic folds to shifts and constants, and only the one butterfly
+// is instantiated).
+template <class R, int DIR, int RADIX, int NS, int M>
 __device__ __forceinline__ void stage_fixed(const cpx<R>* __restrict__ in, cpx<R>* __restrict__ out, int rows,
                                             const cpx<R>* __restrict__ tw) {
   constexpr int nb = M / RADIX;
   constexpr int tstep = M / (NS * RADIX);
-  constexpr int rs = M * LN;
-  const int total = rows * nb * LN;
+  constexpr int rs = M * 18;
+  const int total = rows * nb * 18;
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    const int c = idx % LN;
-    const int q = idx / LN;
+    const int c = idx % 18;
+    const int q = idx / 18;
     const int rr = q / nb, j = q % nb;
     const int kk = j % NS, jq = j / NS;
     const cpx<R>* src = in + rr * rs + c;
     cpx<R> v[RADIX];
-    v[0] = src[j * LN];
+    v[0] = src[j * 18];
 #pragma unroll
     for (int r = 1; r < RADIX; ++r) {
-      const cpx<R> x = src[(j + r * nb) * LN];
-      v[r] = (NS == 1) ? x : cmul(x, twiddle<R, DIR>(tw, r * kk * tstep * TSTRIDE));
+      const cpx<R> x = src[(j + r * nb) * 18];
+      v[r] = (NS == 1) ? x : cmul(x, twiddle<R, DIR>(tw, r * kk * tstep * 2));
     }
-    if constexpr (RADIX == 2) dft2<R, DIR>(v);
-    else if constexpr (RADIX == 3) dft3<R, DIR>(v);
-    else if constexpr (RADIX == 4) dft4<R, DIR>(v);
-    else if constexpr (RADIX == 8) dft8<R, DIR>(v);
-    else dft16<R, DIR>(v);
-    cpx<R>* dst = out + rr * rs + c + (jq * NS * RADIX + kk) * LN;
+    dft<R, DIR, RADIX>(v);
+    cpx<R>* dst = out + rr * rs + c + (jq * NS * RADIX + kk) * 18;
 #pragma unroll
-    for (int r = 0; r < RADIX; ++r) dst[r * NS * LN] = v[r];
+    for (int r = 0; r < RADIX; ++r) dst[r * NS * 18] = v[r];
   }
 }
 
-// Transform every line of an AoS tile; data starts in b0, the result pointer
-// (b0 or b1) is returned.  Ends with a barrier.  `tw`, when given, is a copy
-// of the plan's twiddle table (e.g. in shared memory).
-template <class R, int DIR, int MAXR>
-__device__ cpx<R>* tile_fft(cpx<R>* b0, cpx<R>* b1, int rows, const AxisPlan<R>& p,
-                            const cpx<R>* tw = nullptr) {
+// Transform every line of an AoS tile by the run-time radix plan; data starts in
+// b0, the result pointer (b0 or b1) is returned.  Ends with a barrier.
+template <class R, int DIR>
+__device__ cpx<R>* tile_fft(cpx<R>* b0, cpx<R>* b1, int rows, const RadixPlan& p, const cpx<R>* tw) {
   cpx<R>* in = b0;
   cpx<R>* out = b1;
   int Ns = 1;
-  const cpx<R>* table = tw ? tw : p.tw;
   for (int s = 0; s < p.nstages; ++s) {
-    stage_aos<R, DIR, MAXR>(in, out, rows, p.m, p.radix[s], Ns, table, p.tstride);
+    stage_aos<R, DIR>(in, out, rows, p.m, p.radix[s], Ns, tw);
     Ns *= p.radix[s];
     __syncthreads();
     cpx<R>* t = in;
@@ -390,61 +379,60 @@ __host__ __device__ constexpr XPlan x_plan(int m) {
   }
 }
 
-// The x-axis transform inside pass A (twiddle stride 2: the table holds the
-// N1 = 2 M roots).  Common lengths are unrolled at compile time (radix <= 8,
-// radix 3 last, except 16 x 8 for M = 128 in FP32); others take tile_fft with
-// the host's radix plan.
-template <class R, int DIR>
-__device__ cpx<R>* tile_fft_x(cpx<R>* b0, cpx<R>* b1, int rows, const AxisPlan<R>& p, const cpx<R>* tw) {
+// The forward x transform inside pass A of the lengths whose post-step is a
+// pass of its own: common lengths unrolled at compile time (radix <= 8, radix 3
+// last; 128, 64 and 32 in FP64 only - FP32 fuses their last stage with the
+// post-step), others by the run-time radix plan.
+// (256 is met in FP32 only, but the registers of a 128^3 cell's pass A come out
+// worse with the case outside the switch: 257 -> 265 us.)
+template <class R>
+__device__ cpx<R>* tile_fft_x_fwd(cpx<R>* b0, cpx<R>* b1, int rows, const RadixPlan& p, const cpx<R>* tw) {
   auto sync_swap = [&]() {
     __syncthreads();
     cpx<R>* t = b0;
     b0 = b1;
     b1 = t;
   };
+  if constexpr (sizeof(R) == 8) {
+    switch (p.m) {
+      case 128:
+        stage_fixed<R, -1, 8, 1, 128>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, -1, 4, 8, 128>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, -1, 4, 32, 128>(b0, b1, rows, tw); sync_swap();
+        return b0;
+      case 64:
+        stage_fixed<R, -1, 8, 1, 64>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, -1, 8, 8, 64>(b0, b1, rows, tw); sync_swap();
+        return b0;
+      case 32:
+        stage_fixed<R, -1, 8, 1, 32>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, -1, 4, 8, 32>(b0, b1, rows, tw); sync_swap();
+        return b0;
+      default: break;
+    }
+  }
   switch (p.m) {
     case 256:
-      stage_fixed<R, DIR, 8, 1, 256, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 8, 8, 256, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 4, 64, 256, 2>(b0, b1, rows, tw); sync_swap();
-      return b0;
-    case 128:
-      if constexpr (sizeof(R) == 4) {
-        // two stages (16 x 8): one shared-memory pass and one barrier fewer
-        // (FP64 keeps three: its radix-16 butterfly costs more than it saves)
-        stage_fixed<R, DIR, 16, 1, 128, 2>(b0, b1, rows, tw); sync_swap();
-        stage_fixed<R, DIR, 8, 16, 128, 2>(b0, b1, rows, tw); sync_swap();
-      } else {
-        stage_fixed<R, DIR, 8, 1, 128, 2>(b0, b1, rows, tw); sync_swap();
-        stage_fixed<R, DIR, 4, 8, 128, 2>(b0, b1, rows, tw); sync_swap();
-        stage_fixed<R, DIR, 4, 32, 128, 2>(b0, b1, rows, tw); sync_swap();
-      }
-      return b0;
-    case 64:
-      stage_fixed<R, DIR, 8, 1, 64, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 8, 8, 64, 2>(b0, b1, rows, tw); sync_swap();
-      return b0;
-    case 32:
-      stage_fixed<R, DIR, 8, 1, 32, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 4, 8, 32, 2>(b0, b1, rows, tw); sync_swap();
-      return b0;
-    case 16:
-      stage_fixed<R, DIR, 4, 1, 16, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 4, 4, 16, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 8, 1, 256>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 8, 8, 256>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 4, 64, 256>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 24:
-      stage_fixed<R, DIR, 8, 1, 24, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 3, 8, 24, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 8, 1, 24>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 3, 8, 24>(b0, b1, rows, tw); sync_swap();
+      return b0;
+    case 16:
+      stage_fixed<R, -1, 4, 1, 16>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 4, 4, 16>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 12:
-      stage_fixed<R, DIR, 4, 1, 12, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, DIR, 3, 4, 12, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 4, 1, 12>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 3, 4, 12>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 8:
-      stage_fixed<R, DIR, 8, 1, 8, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, -1, 8, 1, 8>(b0, b1, rows, tw); sync_swap();
       return b0;
-    default:
-      return tile_fft<R, DIR, 8>(b0, b1, rows, p, tw);
+    default: return tile_fft<R, -1>(b0, b1, rows, p, tw);
   }
 }
 

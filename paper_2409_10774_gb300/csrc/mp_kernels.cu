@@ -284,7 +284,7 @@ __device__ __forceinline__ void x_fwd_planned(cpx<R>* z, cpx<R>* other, int rows
 // Inverse x transform of packed rows: the spectral rows X in b0 -> the
 // packed real rows (returned: b0 or b1).  Ends with a barrier.
 template <class R>
-__device__ cpx<R>* tile_fft_x_inv_packed(cpx<R>* b0, cpx<R>* b1, int rows, const AxisPlan<R>& p, int msh,
+__device__ cpx<R>* tile_fft_x_inv_packed(cpx<R>* b0, cpx<R>* b1, int rows, const RadixPlan& p, int msh,
                                          const cpx<R>* tw) {
   auto sync_swap = [&]() {
     __syncthreads();
@@ -295,38 +295,38 @@ __device__ cpx<R>* tile_fft_x_inv_packed(cpx<R>* b0, cpx<R>* b1, int rows, const
   switch (p.m) {
     case 256:
       stage_first_inv_packed<R, 8, 256>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 8, 8, 256, 2>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 4, 64, 256, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 8, 8, 256>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 4, 64, 256>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 128:  // as the forward transform: 16 x 8 in FP32, 8 x 4 x 4 in FP64
       if constexpr (sizeof(R) == 4) {
         stage_first_inv_packed<R, 16, 128>(b0, b1, rows, tw); sync_swap();
-        stage_fixed<R, +1, 8, 16, 128, 2>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, +1, 8, 16, 128>(b0, b1, rows, tw); sync_swap();
       } else {
         stage_first_inv_packed<R, 8, 128>(b0, b1, rows, tw); sync_swap();
-        stage_fixed<R, +1, 4, 8, 128, 2>(b0, b1, rows, tw); sync_swap();
-        stage_fixed<R, +1, 4, 32, 128, 2>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, +1, 4, 8, 128>(b0, b1, rows, tw); sync_swap();
+        stage_fixed<R, +1, 4, 32, 128>(b0, b1, rows, tw); sync_swap();
       }
       return b0;
     case 64:
       stage_first_inv_packed<R, 8, 64>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 8, 8, 64, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 8, 8, 64>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 32:
       stage_first_inv_packed<R, 8, 32>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 4, 8, 32, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 4, 8, 32>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 16:
       stage_first_inv_packed<R, 4, 16>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 4, 4, 16, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 4, 4, 16>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 24:
       stage_first_inv_packed<R, 8, 24>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 3, 8, 24, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 3, 8, 24>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 12:
       stage_first_inv_packed<R, 4, 12>(b0, b1, rows, tw); sync_swap();
-      stage_fixed<R, +1, 3, 4, 12, 2>(b0, b1, rows, tw); sync_swap();
+      stage_fixed<R, +1, 3, 4, 12>(b0, b1, rows, tw); sync_swap();
       return b0;
     case 8:
       stage_first_inv_packed<R, 8, 8>(b0, b1, rows, tw); sync_swap();
@@ -335,7 +335,7 @@ __device__ cpx<R>* tile_fft_x_inv_packed(cpx<R>* b0, cpx<R>* b1, int rows, const
       if (const XPlan P = x_plan(p.m); P.count > 0) return x_inv_planned<R>(b0, b1, rows, p.m, P, tw);
       x_inverse_pre<R>(b0, b1, rows, p.m, msh, tw);
       __syncthreads();
-      return tile_fft<R, +1, 8>(b1, b0, rows, p, tw);
+      return tile_fft<R, +1>(b1, b0, rows, p, tw);
   }
 }
 
@@ -372,7 +372,7 @@ __device__ __forceinline__ void x_forward_last_post(const cpx<R>* __restrict__ i
     const int rr = q / UNITS, u = q - rr * UNITS;
     const cpx<R>* src = in + rr * RS + c;
     cpx<R>* dst = X + rr * RS + c;
-    // butterfly j of the stage (as stage_fixed<R, -1, RADIX, NS, M, 2>)
+    // butterfly j of the stage (as stage_fixed<R, -1, RADIX, NS, M>)
     auto butterfly = [&](int j, cpx<R>(&v)[RADIX]) {
       v[0] = src[j * LN];
 #pragma unroll
@@ -565,7 +565,7 @@ __device__ __forceinline__ bool pass_a_item(const CellDev<R>& c, long long item,
   // shared memory): staged for the block's first item of each cell
   if (reload) {
     if (use_vox && threadIdx.x < 18) tms[threadIdx.x] = (R)c.tmean[threadIdx.x];
-    for (int k = threadIdx.x; k < N1; k += blockDim.x) tws[k] = c.px.tw[k];
+    for (int k = threadIdx.x; k < N1; k += blockDim.x) tws[k] = c.tw[0][k];
   }
   if (threadIdx.x == 0) {
     // the block's next item (single cell), fetched into L2 while this one runs
@@ -866,9 +866,9 @@ __device__ __forceinline__ bool pass_a_item(const CellDev<R>& c, long long item,
     // FP32: the first stage of the compile-time plan, then its last stage
     // fused with the post-step (128: 16 x 8, 64: 8 x 8, 32: 8 x 4)
     cpx<R>* other = (zbuf == b0) ? b1 : b0;
-    if (M == 128) stage_fixed<R, -1, 16, 1, 128, 2>(zbuf, other, nr, tws);
-    else if (M == 64) stage_fixed<R, -1, 8, 1, 64, 2>(zbuf, other, nr, tws);
-    else stage_fixed<R, -1, 8, 1, 32, 2>(zbuf, other, nr, tws);
+    if (M == 128) stage_fixed<R, -1, 16, 1, 128>(zbuf, other, nr, tws);
+    else if (M == 64) stage_fixed<R, -1, 8, 1, 64>(zbuf, other, nr, tws);
+    else stage_fixed<R, -1, 8, 1, 32>(zbuf, other, nr, tws);
     __syncthreads();
     if (M == 128) x_forward_last_post<R, 128, 8>(other, zbuf, nr, tws);
     else if (M == 64) x_forward_last_post<R, 64, 8>(other, zbuf, nr, tws);
@@ -880,7 +880,7 @@ __device__ __forceinline__ bool pass_a_item(const CellDev<R>& c, long long item,
     X = zbuf;
   } else if (packed) {
     cpx<R>* other = (zbuf == b0) ? b1 : b0;
-    cpx<R>* Z = tile_fft_x<R, -1>(zbuf, other, nr, c.px, tws);
+    cpx<R>* Z = tile_fft_x_fwd<R>(zbuf, other, nr, c.px, tws);
     cpx<R>* dst = (Z == b0) ? b1 : b0;
     x_forward_post<R>(Z, dst, nr, M, msh, tws);
     X = dst;
@@ -1180,8 +1180,8 @@ __global__ void __launch_bounds__(kThreads, (sizeof(R) == 4 ? 2 : 1))
   uint32_t parity = 0;
   bool failed = false;
   int* status = c0.status;
-  // the per-thread carries (error maxima and sums, row sums of threads 32..67)
-  // start at zero; they sit after the item buffers for the block's row count
+  // the per-thread carries (error maxima and sums, row sums) start at zero; they
+  // sit after the item buffers for the block's row count
   const PassASmem<R> SL(c0.n1 > 0 ? c0.n1 : 1, c0.rows_a > 0 ? c0.rows_a : 1);
   if constexpr (!MULTI) {
     R* cmx = reinterpret_cast<R*>(smem_raw + SL.carry_off);

@@ -381,7 +381,7 @@ __device__ __forceinline__ void line_tile(const CellDev<R>& c, long long tile, c
   cpx<R>* a = tw + line_table(N);
   cpx<R>* b = a + line_pitch(N, LN) * cols;
   if (fresh) {
-    const cpx<R>* t = PASS < kZReduced ? c.py.tw : c.pz.tw;
+    const cpx<R>* t = PASS < kZReduced ? c.tw[1] : c.tw[2];
     const R f = c.two_pi_over_L[PASS < kZReduced ? 1 : 2];
     for (int k = threadIdx.x; k < N; k += blockDim.x) {
       tw[k] = t[k];
@@ -412,12 +412,21 @@ __global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS, N)
   X(1) X(2) X(4) X(6) X(8) X(12) X(16) X(18) X(24) X(32) X(36) X(48) X(54) X(64) X(72) X(96) X(108) X(128) \
   X(144) X(162) X(192) X(216) X(256) X(288) X(324) X(384) X(432) X(486) X(512)
 
+// Whether a pass meets a length: cells of one y point have no y pass, and FP64
+// columns beyond 384 points do not fit a tile (sizes_fit).
+template <class R>
+__host__ __device__ constexpr bool line_exists(int pass, int n) {
+  return (n > 1 || pass >= kZReduced) && (sizeof(R) == 4 || n <= 384);
+}
+
 // Several cells: the length is dispatched per tile.
 template <class R, int PASS>
 __device__ __forceinline__ void line_tile_any(const CellDev<R>& c, long long tile, cpx<R>* smem, bool fresh) {
   switch (PASS < kZReduced ? c.n2 : c.n3) {
 #define MP_CASE(N) \
-  case N: line_tile<R, PASS, N>(c, tile, smem, fresh); break;
+  case N:                                                                              \
+    if constexpr (line_exists<R>(PASS, N)) line_tile<R, PASS, N>(c, tile, smem, fresh); \
+    break;
     MP_LINE_LENGTHS(MP_CASE)
 #undef MP_CASE
     default: break;  // refused by validation
@@ -441,7 +450,8 @@ __global__ void __launch_bounds__(line_threads<R>(PASS), line_blocks<R>(PASS, 25
 // ------------------------------------------------------------------ launches
 template <class R, int PASS, int N>
 const void* line_kernel() {
-  if constexpr (PASS < kZReduced) return (const void*)k_fft_y<R, PASS, N>;
+  if constexpr (!line_exists<R>(PASS, N)) return nullptr;
+  else if constexpr (PASS < kZReduced) return (const void*)k_fft_y<R, PASS, N>;
   else return (const void*)k_green_z<R, PASS, N>;
 }
 template <class R, int PASS>

@@ -7,7 +7,6 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
-#include <vector>
 
 #include "mp_common.cuh"
 
@@ -47,11 +46,13 @@ inline int tile_columns(int n, long long ncols, bool fp64, bool shared, int nsm)
   return best;
 }
 
-// Radix sequence of the packed x axis' complex transform of length m = 2^a 3^b
+// Radix sequence of the packed x axis' complex transform of length n1 / 2 = 2^a 3^b
 // (for the lengths without compile-time stages): powers of two in as few
 // radix-8 stages as possible, radix-3 stages last.
-inline void radix_plan(int m, int* radix, int& nst) {
-  nst = 0;
+inline RadixPlan radix_plan(int n1) {
+  RadixPlan p{};
+  p.m = n1 > 1 ? n1 / 2 : 1;
+  int m = p.m;
   int k2 = 0;
   while (m % 2 == 0) {
     m /= 2;
@@ -64,53 +65,38 @@ inline void radix_plan(int m, int* radix, int& nst) {
   }
   static const int kPlan2[10][3] = {{0}, {2}, {4}, {8}, {4, 4}, {8, 4}, {8, 8}, {8, 4, 4}, {8, 8, 4}, {8, 8, 8}};
   static const int kLen2[10] = {0, 1, 1, 1, 2, 2, 2, 3, 3, 3};
-  for (int i = 0; i < kLen2[k2]; ++i) radix[nst++] = kPlan2[k2][i];
-  for (int i = 0; i < k3; ++i) radix[nst++] = 3;
+  for (int i = 0; i < kLen2[k2]; ++i) p.radix[p.nstages++] = kPlan2[k2][i];
+  for (int i = 0; i < k3; ++i) p.radix[p.nstages++] = 3;
+  return p;
 }
 
-// FFT plan of one axis and its twiddle table, computed in FP64 and rounded to
-// R (host_tw receives n entries; p.tw is left for the caller to point at the
-// device copy).  packed: the x axis, a real transform of length n through a
-// complex one of length n / 2.
+// Twiddle table of an axis, computed in FP64 and rounded to R (n entries).
 template <class R>
-void axis_plan(int n, bool packed, AxisPlan<R>& p, cpx<R>* host_tw) {
-  p.n = n;
-  p.m = packed ? (n > 1 ? n / 2 : 1) : n;
-  p.tstride = packed ? 2 : 1;
-  p.nstages = 0;  // the y / z lines have compile-time plans (line_plan)
-  if (packed) radix_plan(p.m, p.radix, p.nstages);
+void twiddle_table(int n, cpx<R>* tw) {
   for (int k = 0; k < n; ++k) {
     const double a = 2.0 * M_PI * (double)k / (double)n;
-    host_tw[k].x = (R)std::cos(a);
-    host_tw[k].y = (R)(-std::sin(a));
+    tw[k].x = (R)std::cos(a);
+    tw[k].y = (R)(-std::sin(a));
   }
-  p.tw = nullptr;
 }
 
 // What a Green-operator call uploads, as one image: `words` zeroed 32-bit words
 // (status and control), then the three axes' twiddle tables, 16-byte aligned.
-// Fills `image` (kImageBytes), the plans and the tables' byte offsets (the
-// plans' tw pointers are base + table[a]); returns the image's size.
+// Fills `image` (kImageBytes) and the tables' byte offsets; returns the image's
+// size.
 constexpr size_t kImageBytes = 32 * 1024;
 template <class R>
-size_t operator_image(const int32_t n[3], AxisPlan<R>* const plan[3], size_t words, unsigned char* image,
-                      size_t table[3]) {
+size_t operator_image(const int32_t n[3], size_t words, unsigned char* image, size_t table[3]) {
   size_t o = (words * 4 + 15) / 16 * 16;
   std::memset(image, 0, o);
   for (int a = 0; a < 3; ++a) {
     table[a] = o;
-    axis_plan<R>(n[a], a == 0, *plan[a], reinterpret_cast<cpx<R>*>(image + o));
+    twiddle_table<R>(n[a], reinterpret_cast<cpx<R>*>(image + o));
     o += ((size_t)n[a] * sizeof(cpx<R>) + 15) / 16 * 16;
   }
   return o;
 }
 static_assert(4 * (4 + 2 + 2 * 256) + 16 + 3 * 512 * sizeof(cpx<double>) <= kImageBytes,
               "the largest image: control words of 256 kx planes, three axes of 512 points");
-
-template <class R>
-void axis_tables(int n, bool packed, AxisPlan<R>& p, std::vector<cpx<R>>& host_tw) {
-  host_tw.resize(n);
-  axis_plan<R>(n, packed, p, host_tw.data());
-}
 
 }  // namespace mp

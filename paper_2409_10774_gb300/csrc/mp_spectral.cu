@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_spectral(CellDev<float> c, int* c
   uint64_t* full = reinterpret_cast<uint64_t*>(tw + kN);                       // [kStages]
   uint64_t* empty = full + kStages;                                             // [kStages]
   SlotInfo* info = reinterpret_cast<SlotInfo*>(empty + kStages);               // [kStages]
-  for (int k = threadIdx.x; k < kN; k += blockDim.x) tw[k] = c.py.tw[k];
+  for (int k = threadIdx.x; k < kN; k += blockDim.x) tw[k] = c.tw[1][k];
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mb_init(&full[s], 33);  // the producer's 32 lanes once their copies have landed, + lane 0's slot info

@@ -100,12 +100,12 @@ mp_status run(mp_ctx* ctx, const int32_t n[3], double h, const double ref[6], co
   c.spec = reinterpret_cast<cpx<R>*>(b + kTableRegion);
   c.status = reinterpret_cast<int*>(b);
   // status word and twiddle tables W_N^k = exp(-2 pi i k / N), uploaded as one image
-  AxisPlan<R>* const plans[3] = {&c.px, &c.py, &c.pz};
+  c.px = radix_plan(c.n1);
   static thread_local __align__(16) unsigned char image[kImageBytes];
   static_assert(kImageBytes <= kTableRegion, "the image fits its region");
   size_t table[3];
-  const size_t image_bytes = operator_image<R>(n, plans, 4, image, table);  // the plans every entry point uses
-  for (int a = 0; a < 3; ++a) plans[a]->tw = reinterpret_cast<const cpx<R>*>(b + table[a]);
+  const size_t image_bytes = operator_image<R>(n, 4, image, table);
+  for (int a = 0; a < 3; ++a) c.tw[a] = reinterpret_cast<const cpx<R>*>(b + table[a]);
   cudaError_t e = cudaMemcpyAsync(b, image, image_bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     LaunchCfg L = make_launch_cfg<R>(c, ctx->nsm > 0 ? ctx->nsm : 1);
