@@ -27,7 +27,8 @@
  *         means and ratios (eq. err) in FP64 (the per-voxel norms of FP32
  *         field differences are FP32 quantities and their maxima are exact),
  *         and the homogenized averages accumulated in compensated FP32
- *         pairs (per thread) and folded in FP64 (p, q summed in FP64).
+ *         pairs (per thread; batched cells' in FP64) and folded in FP64 (p, q
+ *         summed in FP64).
  *         Without a prescribed iteration schedule or a manufactured source, an
  *         increment whose error sets no new low (below 0.99 times the last
  *         one) in 64 iterations while above the tolerance (the FP32

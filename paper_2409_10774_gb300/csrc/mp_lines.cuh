@@ -22,10 +22,10 @@
 // pass; their z pass takes all 18.
 //
 // Every supported length has a compile-time plan of one to three Stockham
-// stages (radices up to 18, the coprime ones without twiddles).  The first
-// stage reads global memory straight into registers and the last one of the
-// passes that end in all lines stores from registers, so a two-stage pass
-// crosses shared memory twice.  Tiles are whole columns: (col N + p) LN + c.
+// stages (radices up to 18, the coprime ones without twiddles).  Tiles are whole
+// columns, (col N + p) LN + c, loaded into shared memory in 16-byte asynchronous
+// copies; the last stage of the y inverse and z passes stores to global memory
+// from registers.
 #pragma once
 
 #include "mp_device.cuh"
